@@ -235,10 +235,14 @@ void mdbs_batch_destroy(mdbs_batch* batch);
  *   smooth_rows : 1, 2, 4 or 8 rows of 256 cells per CTA work item in the
  *                 finest-level red-black sweeps (fewer rows: more CTAs in flight)
  *   tail_cells  : 0 .. 262144; levels with at most this many cells run, with all
- *                 coarser ones, inside one kernel with tail_ctas CTAs per domain
- *                 (fewer launches, less parallelism)
- *   tail_ctas   : 1, 2, 4 or 8; CTAs of 1024 threads per domain in that kernel (more
- *                 than one: a thread-block cluster synchronised by cluster barriers)
+ *                 coarser ones, inside one kernel (fewer launches, less parallelism).
+ *                 Where that starts at a level of at most 4096 cells in every domain,
+ *                 the kernel is a thread-block cluster per domain that keeps the levels
+ *                 in its shared memory; a domain that lies wholly in it, of at most
+ *                 4096 cells, runs its whole CG solve there
+ *   tail_ctas   : 1, 2, 4 or 8; CTAs per domain in that kernel (more than one: a
+ *                 thread-block cluster synchronised by cluster barriers); 1 leaves the
+ *                 size of the clusters above to the library
  *   snake       : 0 or 1; 1 alternates the traversal direction of consecutive
  *                 kernels over one level, so each starts on the cache lines the
  *                 previous one touched last

@@ -2,6 +2,7 @@
 // every launch's flat block index to (domain, local block), and the device
 // tables of per-domain views.  Built once per batch composition.
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #include "mdbs_internal.cuh"
@@ -37,8 +38,19 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
     if (e != cudaSuccess) return e;
   }
   // host block tables: spaces in a fixed order, each ndom + 1 prefix entries
-  const int nspace = 5 + 6 * kMaxLevels;
-  std::vector<int> tab((size_t)nspace * (ndom + 1), 0);
+  const int nspace = 6 + 7 * kMaxLevels;  // the last one: CG vectors
+  const int scg = nspace - 1;
+  // after the spaces: the indexes of the small domains, then of the others
+  std::vector<int> tab((size_t)nspace * (ndom + 1) + ndom, 0);
+  int* const idx = &tab[(size_t)nspace * (ndom + 1)];
+  for (int d = 0; d < ndom; d++)
+    if (cg[d].small) idx[B.n_small++] = d;
+  for (int d = 0; d < ndom; d++)
+    if (!cg[d].small) idx[B.n_small + B.n_big++] = d;
+  {
+    cudaError_t e = plan_clusters(cg, ndom, flexible, tail_ctas, sms, &B);
+    if (e != cudaSuccess) return e;
+  }
   auto fill = [&](int space, auto count) -> int {
     int* t = &tab[(size_t)space * (ndom + 1)];
     long long acc = 0;
@@ -49,11 +61,11 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
     t[ndom] = (int)acc;
     return (int)acc;
   };
-  int totals[5 + 6 * kMaxLevels];
+  int totals[6 + 7 * kMaxLevels];
   // one row of kBlock elements per item, except the reduction spaces (kRepBig rows:
   // fewer block reductions and partials)
-  int reps[5 + 6 * kMaxLevels];
-  for (int q = 0; q < 5 + 6 * kMaxLevels; q++) reps[q] = 1;
+  int reps[6 + 7 * kMaxLevels];
+  for (int q = 0; q < nspace; q++) reps[q] = 1;
   reps[3] = reps[4] = kRepBig;
   reps[5 + kMaxLevels] = smooth_rows;  // finest-level red/black half sweeps
   auto blocks_of = [&](long long n, int space) { return items_of(n, reps[space]); };
@@ -62,6 +74,7 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
   totals[2] = fill(2, [&](int) { return 1LL; });
   totals[3] = fill(3, [&](int d) { return blocks_of(sd[d].P.cells, 3); });
   totals[4] = fill(4, [&](int d) { return blocks_of(faces_total(sd[d].P), 4); });
+  totals[scg] = fill(scg, [&](int d) { return cg[d].small ? 0LL : cg_items(sd[d].P.cells); });
   B.max_first = 0;
   B.max_levels = 0;
   B.any_cfl = 0;
@@ -108,6 +121,10 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
       const long long halfs = (long long)(L.n[0] / 2) * L.n[1] * L.n[2];
       return (halfs / V + kBlock - 1) / kBlock;
     });
+    const int s6 = 5 + 6 * kMaxLevels + l;
+    totals[s6] = fill(s6, [&](int d) -> long long {
+      return l < cg[d].first ? (cells_at(d, l + 1) + kBlock / 4 - 1) / (kBlock / 4) : 0LL;
+    });
     const int s4 = 5 + 4 * kMaxLevels + l;
     totals[s4] = fill(s4, [&](int d) -> long long {
       if (l >= cg[d].first || sweep_kz <= 0) return 0;
@@ -123,7 +140,23 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
   if (e == cudaSuccess) e = cudaMemcpy(B.sd, sd, ndom * sizeof(StepDom), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&B.cg, ndom * sizeof(CgDom));
   if (e == cudaSuccess) e = cudaMemcpy(B.cg, cg, ndom * sizeof(CgDom), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&B.any_flag, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&B.any_flag, 2 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(B.any_flag, 0, 2 * sizeof(int));
+  std::vector<CgVec> cv(ndom);
+  for (int d = 0; d < ndom; d++) {
+    const Prm& P = sd[d].P;
+    const Fld& F = sd[d].F;
+    const CgDom& G = cg[d];
+    cv[d] = CgVec{{P.n[0], P.n[1], P.n[2]}, (unsigned)P.cells, P.dn0, P.dn1, G.r, G.z, G.dv, G.q, F.p,
+                  F.b, F.diag, {F.T[0], F.T[1], F.T[2]}, G.lf[0].b, G.lf[0].x, G.partials, G.pcap, G.scal};
+  }
+  if (e == cudaSuccess) e = cudaMalloc(&B.cv, ndom * sizeof(CgVec));
+  if (e == cudaSuccess) e = cudaMemcpy(B.cv, cv.data(), ndom * sizeof(CgVec), cudaMemcpyHostToDevice);
+  B.one_cv = cv[0];
+  if (e == cudaSuccess && ndom == 1) {
+    B.one_cg = new (std::nothrow) CgDom(cg[0]);
+    if (!B.one_cg) e = cudaErrorMemoryAllocation;
+  }
   if (e == cudaSuccess) e = cudaMalloc(&B.err_flag, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(B.err_flag, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&B.coop_ctr, sizeof(unsigned long long));
@@ -146,6 +179,9 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
   B.dom = work(2);
   B.rcells = work(3);
   B.rfaces = work(4);
+  B.cgcells = work(scg);
+  B.small_idx = B.table_storage + (size_t)nspace * (ndom + 1);
+  B.big_idx = B.small_idx + B.n_small;
   for (int l = 0; l < kMaxLevels; l++) {
     B.lcells[l] = work(5 + l);
     B.lhalf[l] = work(5 + kMaxLevels + l);
@@ -153,6 +189,7 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
     B.lcoarse[l] = work(5 + 3 * kMaxLevels + l);
     B.lsweep[l] = work(5 + 4 * kMaxLevels + l);
     B.lvec[l] = work(5 + 5 * kMaxLevels + l);
+    B.lrest[l] = work(5 + 6 * kMaxLevels + l);
   }
   *out = B;
   return cudaSuccess;
@@ -162,6 +199,10 @@ void plan_destroy(BatchPlan* B) {
   if (B->table_storage) cudaFree(B->table_storage);
   if (B->sd) cudaFree(B->sd);
   if (B->cg) cudaFree(B->cg);
+  if (B->cv) cudaFree(B->cv);
+  delete B->one_cg;
+  B->cv = nullptr;
+  B->one_cg = nullptr;
   if (B->any_flag) cudaFree(B->any_flag);
   if (B->err_flag) cudaFree(B->err_flag);
   if (B->coop_ctr) cudaFree(B->coop_ctr);

@@ -154,7 +154,8 @@ struct CgDom {
   Level<double> ld[kMaxLevels];  // FP64 hierarchy (level 0 arrays point into Fld)
   Level<float> lf[kMaxLevels];   // FP32 hierarchy (mixed precision)
   int nlev;
-  int first;  // first level handled by the single-CTA tail
+  int first;  // first level handled by the tail kernel
+  int small;  // the whole CG solve runs in one cluster
   double *r, *z, *dv, *q;
   double* partials;  // 2 channels of pcap values
   long long pcap;
@@ -166,6 +167,24 @@ struct CgDom {
   const CUtensorMap* tmaps;
   unsigned tma_levels;
 };
+
+// what the CG vector kernels need of a domain; passed by value to a kernel that runs over a
+// single domain (the pointers then come from the constant bank instead of two dependent loads)
+struct CgVec {
+  int n[3];
+  unsigned cells;
+  FastDiv dn0, dn1;
+  double *r, *z, *dv, *q, *p;
+  const double *b, *diag, *T[3];
+  float *bf;         // FP32 V-cycle's right-hand side and result (mixed precision)
+  const float* xf;
+  double* partials;
+  long long pcap;
+  double* scal;
+};
+
+// partial sums of a domain's CG reductions: kRepBig rows of kBlock cells each
+inline long long cg_items(long long cells) { return (cells + kBlock * kRepBig - 1) / (kBlock * kRepBig); }
 
 // ---------------------------------------------------------------- helpers
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
@@ -200,7 +219,8 @@ __device__ __forceinline__ double block_sum(double v) {
   int nw = (blockDim.x + 31) >> 5;
   v = (threadIdx.x < nw) ? warp_part[threadIdx.x] : 0.0;
   if (w == 0)
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < nw) v += __shfl_down_sync(0xffffffffu, v, o);  // beyond nw only zeros would be added
   return v;
 }
 
@@ -234,7 +254,7 @@ enum KernelId {
   K_ALPHA_FLUX, K_ALPHA_LO, K_ALPHA_LIMIT, K_ALPHA_UPDATE, K_FINALIZE, K_PROPERTIES, K_NORMALS,
   K_CURVATURE, K_MOM_ASSEMBLE, K_JACOBI, K_HBYA, K_CORRECT, K_BOUNDARY, K_STATS, K_CFL, K_STATIC,
   K_ASSEMBLE, K_DIAG, K_CONVERT, K_COARSEN, K_SMOOTH0, K_SMOOTHC, K_ZERO, K_RESTRICT0, K_RESTRICTC,
-  K_PROLONG0, K_PROLONGC, K_RESID0, K_SPMV_DOT, K_UPDATE_XR, K_DOTS, K_UPDATE_D, K_TAIL, K_COOP, K_EDGE_MU, K_COUNT
+  K_PROLONG0, K_PROLONGC, K_RESID0, K_SPMV_DOT, K_UPDATE_XR, K_DOTS, K_UPDATE_D, K_TAIL, K_COOP, K_EDGE_MU, K_CG_CLUSTER, K_COUNT
 };
 extern const char* const kKernelNames[K_COUNT];
 void prof_begin(int id, cudaStream_t s);
@@ -257,6 +277,14 @@ long long launch_count();  // kernels launched so far by the active simulation
     asm volatile("griddepcontrol.wait;\n" ::: "memory");          \
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); \
   } while (0)
+
+// The two halves apart, for the kernels of the CG loop: they let their successor launch at
+// once and read what no kernel of the loop writes (tables, coefficients, reciprocal
+// diagonals: written by the operator's build, which has completed before the loop's first
+// kernel starts) before they wait.  A kernel that has not waited may run beside any number
+// of its predecessors, so it must touch nothing else.
+#define MDBS_PDL_TRIGGER() asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory")
+#define MDBS_PDL_WAIT() asm volatile("griddepcontrol.wait;\n" ::: "memory")
 
 #define MDBS_LAUNCH_SMEM(ID, GRID, BLOCK, SMEM, STREAM, KERNEL, ...)                                \
   do {                                                                                             \
@@ -287,10 +315,18 @@ struct BatchPlan {
   int grid_cap;               // persistent grid: SMs x resident blocks
   Work cells, faces, dom;     // per-domain cells, faces (one row per item), one block per domain
   Work rcells, rfaces;        // the same with kRepBig rows per item: kernels with block reductions
+  Work cgcells;               // CG vectors: kRepBig rows per item, domains solved by clusters left out
+  int n_small, n_big;         // domains whose CG solve runs in a cluster, and the others
+  const int *small_idx, *big_idx;  // device: their indexes
+  int small_rows, small_ctas; // reduction rows per CTA and CTAs per cluster of the CG kernel,
+  size_t small_smem;          // its dynamic shared memory
+  int cl_tail_ctas;           // > 0: the tails run in clusters of this many CTAs
+  size_t cl_tail_smem;
   Work lcells[kMaxLevels];    // level-l cells of domains that have level l
   Work lhalf[kMaxLevels];     // level-l red/black half cells of domains whose level l precedes the tail
   Work lfine[kMaxLevels];     // level-l cells of the same domains (prolongation)
-  Work lcoarse[kMaxLevels];   // level-(l+1) cells of the same domains (restriction)
+  Work lcoarse[kMaxLevels];   // level-(l+1) cells of the same domains (restriction phase of the cooperative kernel)
+  Work lrest[kMaxLevels];     // the same in items of kBlock / 4 cells (the restriction's launches)
   Work lsweep[kMaxLevels];    // fused-sweep tiles (kSweepTX x kSweepTY columns x sweep_kz planes) of the same domains
   Work lvec[kMaxLevels];      // vector half sweeps: kBlock threads x (2 FP64 / 4 FP32) half cells per item
   unsigned vec_levels;        // bit l: every domain's level l (before its tail) allows vector half sweeps
@@ -308,8 +344,11 @@ struct BatchPlan {
   unsigned long long* coop_ctr;  // device: arrival counter of its grid barriers
   StepDom* sd;                // device tables (ndom entries)
   CgDom* cg;
+  CgVec* cv;
+  CgDom* one_cg;              // host copies, for kernels over a single domain (ndom == 1)
+  CgVec one_cv;
   int* table_storage;         // device memory of every block table
-  int* any_flag;              // device: some domain still iterating (CG WHILE condition)
+  int* any_flag;              // device: some domain still iterating (CG WHILE condition); [1] arrivals
   int* err_flag;              // device: a kernel's bounded wait ran out (the batch's results are invalid)
 };
 
@@ -392,6 +431,8 @@ cudaError_t bounded_wait_selftest(int* status, double* waited_s);
 // coarse_coop: run the levels between the finest and the tail in one cooperative launch
 cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexible, int smooth_rows, int snake,
                         int sweep_kz, int tail_ctas, int coarse_coop, int vec_sweeps, BatchPlan* out);
+// launch shape of the cluster kernels (pressure.cu); n_small / n_big are set
+cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas, int sms, BatchPlan* B);
 // CTAs of the cooperative coarse-level kernel that are resident at once on this device
 cudaError_t coop_grid_size(int flexible, long long tail_words, int* grid);
 void plan_destroy(BatchPlan* B);

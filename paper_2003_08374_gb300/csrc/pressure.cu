@@ -9,8 +9,10 @@
 #include <cudaTypedefs.h>  // PFN_cuTensorMapEncodeTiled
 #include <cuda_bf16.h>
 #include <math.h>
+#include <stddef.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -120,7 +122,7 @@ __device__ __forceinline__ void with_coefs(const Level<R>& L, F&& f) {
 }
 
 // CG scalars on the device
-constexpr int kBB = 0, kRR = 1, kRZ = 2, kDQ = 3, kZQ = 4, kAlpha = 5, kCond = 6, kRZold = 7, kIt = 8;
+constexpr int kBB = 0, kRR = 1, kRZ = 2, kDQ = 3, kZQ = 4, kAlpha = 5, kCond = 6, kBeta = 7, kIt = 8;
 
 #define FOR_WORK(W)                                   \
   for (int b_ = blockIdx.x; b_ < (W).total; b_ += gridDim.x) { \
@@ -276,7 +278,6 @@ __global__ void k_coarsen(const CgDom* __restrict__ C, Work w, int l) {
   }
 }
 
-// sum_nb T x_nb at cell c of level L (order x-, x+, y-, y+, z-, z+)
 // Load of an iterate or right-hand side.  COH: through L2 (ld.global.cg), for the
 // phases of the cooperative kernel, where other CTAs rewrote the value since this
 // SM may last have read it (L2 is the point of coherence; a load that allocates in
@@ -289,23 +290,29 @@ __device__ __forceinline__ R ldc(const R* p) {
     return *p;
 }
 
-template <typename R, bool COH = false>
-__device__ __forceinline__ R neighbour_sum(const Level<R>& L, const R* x, const int q[3], long long c) {
-  R v = R(0);
-  for (int d = 0; d < 3; d++) {
-    if (q[d] > 0) {
-      const unsigned cl = lo_pos(L.n, q, (unsigned)c, d);
-      v += tcoef(L, d, cl) * ldc<COH>(x + cl);
-    }
-    if (q[d] + 1 < L.n[d]) v += tcoef(L, d, (unsigned)c) * ldc<COH>(x + hi_pos(L.n, q, (unsigned)c, d));
-  }
-  return v;
-}
-
 // fused multiply-add of the level's precision (every smoother spells out the same
 // fma chain, so no value depends on the compiler's contraction choices)
 __device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
+// a product that is rounded by itself
+__device__ __forceinline__ double mul_r(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b); }
+
+// b - A x at cell q (position c): the neighbour products in the order x-, x+, y-, y+, z-,
+// z+ from zero, then b - (diag x - sum) with the product rounded
+template <typename R, bool COH = false>
+__device__ __forceinline__ R resid_cell(const Level<R>& L, const R* x, const R* b, const int q[3], long long c) {
+  R v = R(0);
+  for (int d = 0; d < 3; d++) {
+    if (q[d] > 0) {
+      const unsigned cl = lo_pos(L.n, q, (unsigned)c, d);
+      v = fma_r(tcoef(L, d, cl), ldc<COH>(x + cl), v);
+    }
+    if (q[d] + 1 < L.n[d])
+      v = fma_r(tcoef(L, d, (unsigned)c), ldc<COH>(x + hi_pos(L.n, q, (unsigned)c, d)), v);
+  }
+  return ldc<COH>(b + c) - (mul_r(L.diag[c], ldc<COH>(x + c)) - v);
+}
 
 // One red-black Gauss-Seidel update of cell c = (i, j, k):
 // x_c = (b_c + sum_nb T x_nb) / diag_c, neighbours in the order x-, x+, y-, y+,
@@ -413,6 +420,100 @@ __global__ void __launch_bounds__(kBlock, REP == 1 ? 8 : 1)
     const CgDom& G = C[dm];
     if (G.scal[kCond] == 0.0) continue;
     smooth_item<R, REP, PRO>(G, l, lb, threadIdx.x, col, zero);
+  }
+}
+
+// two consecutive levels of a domain
+template <typename R>
+struct LvPair {
+  Level<R> fine, coarse;
+};
+
+// The half sweep with one cell a thread.  Everything static -- the cell's position, its six
+// coefficients, its reciprocal diagonal -- is in registers before the wait on the preceding
+// kernel, so what remains after it is one round of loads, the fma chain and the store; a
+// kernel's successors fetch their coefficients while its last blocks finish.  For a single
+// domain: its levels are passed by value (their pointers are in the constant bank), and the
+// loop it runs in is its own (no flag to test).  A batch keeps k_smooth, whose blocks leave
+// a converged domain before they load anything: prefetching made its fine sweeps 45 us
+// where k_smooth takes 34 (16 uneven domains, 4.7 M cells).
+template <typename R, bool PRO>
+__global__ void __launch_bounds__(kBlock, PRO && sizeof(R) == 8 ? 4 : 5)
+    k_sweep(const __grid_constant__ LvPair<R> one, int items, int col, int zero, int rev) {
+  MDBS_PDL_TRIGGER();
+  const Level<R>& L = one.fine;
+  bool waited = false;
+  for (int i_ = blockIdx.x; i_ < items; i_ += gridDim.x) {
+    const int lb = rev ? items - 1 - i_ : i_;
+    const int n0 = L.n[0], n1 = L.n[1], n2 = L.n[2];
+    const unsigned half = (unsigned)(n0 + 1) >> 1, total = half * (unsigned)n1 * (unsigned)n2;
+    const unsigned t = (unsigned)lb * kBlock + threadIdx.x;
+    const unsigned row = fastdiv(t, L.dhalf), ti = t - row * half;
+    const unsigned kk = fastdiv(row, L.dn1);
+    const int j = (int)(row - kk * (unsigned)n1), k = (int)kk;
+    const int sh = (j + k + col) & 1, i = sh + 2 * (int)ti;
+    const bool in = t < total && i < n0;
+    const unsigned sy = (unsigned)n0, sz = (unsigned)n0 * (unsigned)n1;
+    const unsigned rb = sy * row, c = rb + (sh ? half + ti : ti);
+    const unsigned cm = sh ? rb + ti : rb + half + ti - 1, cp = sh ? rb + ti + 1 : rb + half + ti;
+    const bool xm = in && i > 0, xp = in && i + 1 < n0, ym = in && j > 0, yp = in && j + 1 < n1, zm = in && k > 0,
+               zp = in && k + 1 < n2;
+    R di = R(0), t0 = R(0), t1 = R(0), t2 = R(0), t3 = R(0), t4 = R(0), t5 = R(0);
+    if (in) di = L.dinv[c];
+    if (!zero)
+      with_coefs(L, [&](auto Tx, auto Ty, auto Tz) {
+        if (xm) t0 = Tx[cm];
+        if (xp) t1 = Tx[c];
+        if (ym) t2 = Ty[c - sy];
+        if (yp) t3 = Ty[c];
+        if (zm) t4 = Tz[c - sz];
+        if (zp) t5 = Tz[c];
+      });
+    if (!waited) {
+      MDBS_PDL_WAIT();
+      waited = true;
+    }
+    if (!in) continue;
+    R* __restrict__ x = L.x;
+    R v = L.b[c];
+    if (!zero) {
+      R x0 = R(0), x1 = R(0), x2 = R(0), x3 = R(0), x4 = R(0), x5 = R(0);
+      if (xm) x0 = x[cm];
+      if (xp) x1 = x[cp];
+      if (ym) x2 = x[c - sy];
+      if (yp) x3 = x[c + sy];
+      if (zm) x4 = x[c - sz];
+      if (zp) x5 = x[c + sz];
+      if constexpr (PRO) {
+        // the neighbours' corrections (see smooth_cell_corr)
+        const Level<R>& Co = one.coarse;
+        const R* __restrict__ ex = Co.x;
+        const int a = Co.cz[0], b = Co.cz[1], d = Co.cz[2];
+        const unsigned m0 = (unsigned)Co.n[0], m01 = m0 * (unsigned)Co.n[1], he = (m0 + 1) >> 1;
+        const unsigned py = m0 * (unsigned)(j >> b), pz = m01 * (unsigned)(k >> d), px = xs_px(he, i >> a);
+        R e0 = R(0), e1 = R(0), e2 = R(0), e3 = R(0), e4 = R(0), e5 = R(0);
+        if (xm) e0 = ex[py + pz + xs_px(he, (i - 1) >> a)];
+        if (xp) e1 = ex[py + pz + xs_px(he, (i + 1) >> a)];
+        if (ym) e2 = ex[m0 * (unsigned)((j - 1) >> b) + pz + px];
+        if (yp) e3 = ex[m0 * (unsigned)((j + 1) >> b) + pz + px];
+        if (zm) e4 = ex[py + m01 * (unsigned)((k - 1) >> d) + px];
+        if (zp) e5 = ex[py + m01 * (unsigned)((k + 1) >> d) + px];
+        x0 += e0;
+        x1 += e1;
+        x2 += e2;
+        x3 += e3;
+        x4 += e4;
+        x5 += e5;
+      }
+      // in the order of smooth_cell; a missing neighbour's term is left out
+      if (xm) v = fma_r(t0, x0, v);
+      if (xp) v = fma_r(t1, x1, v);
+      if (ym) v = fma_r(t2, x2, v);
+      if (yp) v = fma_r(t3, x3, v);
+      if (zm) v = fma_r(t4, x4, v);
+      if (zp) v = fma_r(t5, x5, v);
+    }
+    x[c] = v * di;
   }
 }
 
@@ -904,26 +1005,104 @@ __device__ __forceinline__ void b_resid_restrict(const Level<R>& Fi, const Level
         if (mask && ((x + y + z) & 1)) continue;
         const int q[3] = {x, y, z};
         const long long c = lpos(Fi.n, x, y, z);
-        const R ax = Fi.diag[c] * ldc<COH>(Fi.x + c) - neighbour_sum<R, COH>(Fi, Fi.x, q, c);
-        s += ldc<COH>(Fi.b + c) - ax;
+        s += resid_cell<R, COH>(Fi, Fi.x, Fi.b, q, c);
       }
   Co.b[ci] = s;
   if (fold && !((Q[0] + Q[1] + Q[2]) & 1)) Co.x[ci] = s * Co.dinv[ci];
 }
 
-template <typename R>
-__global__ void k_resid_restrict(const CgDom* __restrict__ C, Work w, int l, int rev, int sel, int mask, int fold) {
-  MDBS_DEPENDENT_ENTRY();
-  FOR_WORK_DIR(w, rev)
-    const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
-    const Level<R>* L = levels_of<R>(G);
-    Level<R> Fi = L[l];
-    if (sel) Fi.x = Fi.x2;  // the buffer holding the fine iterate
-    for (int r = 0; r < w.rep; r++) {
-      const long long c = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
-      if (c < L[l + 1].cells) b_resid_restrict(Fi, L[l + 1], c, mask, fold);
+// The restriction as a launch: kRestCells coarse cells per item, four threads each.  Thread
+// group g forms the residual of the child with (y, z) offset (g & 1, g >> 1) -- of colour 0
+// alone, one x then fits; without the mask, both -- and the first group sums them in
+// b_resid_restrict's order.  One thread a coarse cell walked its children one after another,
+// four rounds of dependent loads and 36 FP64 instructions of 64 cycles each on the few warps
+// of a coarse level: 20 us for a level of 16^3, however small (cold, ncu).
+constexpr int kRestCells = 64;
+
+template <typename R, bool ONE>
+__global__ void __launch_bounds__(kBlock, 4)
+    k_resid_restrict(const __grid_constant__ LvPair<R> one, const CgDom* __restrict__ C, Work w, int l, int rev,
+                     int sel, int mask, int fold) {
+  static_assert(kBlock == 4 * kRestCells, "four threads a coarse cell");
+  __shared__ R s_res[2][4][kRestCells];
+  MDBS_PDL_TRIGGER();
+  bool waited = false;
+  if (!ONE) {
+    MDBS_PDL_WAIT();
+    waited = true;
+  }
+  const int t = threadIdx.x % kRestCells, g = threadIdx.x / kRestCells;
+  for (int i_ = blockIdx.x; i_ < w.total; i_ += gridDim.x) {
+    const int b_ = rev ? w.total - 1 - i_ : i_;
+    const int dm = ONE ? 0 : work_domain(w, b_);
+    const int lb = ONE ? b_ : b_ - w.blk[dm];
+    if (!ONE && C[dm].scal[kCond] == 0.0) continue;
+    const Level<R>& Fi = ONE ? one.fine : levels_of<R>(C[dm])[l];
+    const Level<R>& Co = ONE ? one.coarse : levels_of<R>(C[dm])[l + 1];
+    const long long ci = (long long)lb * kRestCells + t;
+    const bool in = ci < Co.cells;
+    int Q[3] = {0, 0, 0};
+    if (in) decode_pos(Co, ci, Q[0], Q[1], Q[2]);
+    const int n0 = Fi.n[0], n1 = Fi.n[1], n2 = Fi.n[2];
+    const unsigned sy = (unsigned)n0, sz = (unsigned)n0 * (unsigned)n1, he = (unsigned)(n0 + 1) >> 1;
+    const int dy = g & 1, dz = g >> 1;
+    const int Y = Co.cz[1] ? 2 * Q[1] + dy : Q[1], Z = Co.cz[2] ? 2 * Q[2] + dz : Q[2];
+    const bool pair = in && (Co.cz[1] || !dy) && (Co.cz[2] || !dz) && Y < n1 && Z < n2;
+    const int x_lo = Co.cz[0] ? 2 * Q[0] : Q[0];
+    const int reps = mask ? 1 : 2;
+    const R* __restrict__ x = sel ? Fi.x2 : Fi.x;
+    for (int q = 0; q < reps; q++) {
+      // mask: the x of colour 0 in this row of the coarse cell
+      const int X = x_lo + (mask ? (Co.cz[0] ? (x_lo + Y + Z) & 1 : 0) : q);
+      const bool has = pair && X < n0 && (Co.cz[0] || (mask ? ((X + Y + Z) & 1) == 0 : q == 0));
+      const unsigned rb = sy * (unsigned)Y + sz * (unsigned)Z, c = rb + xs_px(he, X);
+      const unsigned cm = rb + xs_px(he, X - 1), cp = rb + xs_px(he, X + 1);
+      const bool xm = has && X > 0, xp = has && X + 1 < n0, ym = has && Y > 0, yp = has && Y + 1 < n1, zm = has && Z > 0,
+                 zp = has && Z + 1 < n2;
+      R dg = R(0), t0 = R(0), t1 = R(0), t2 = R(0), t3 = R(0), t4 = R(0), t5 = R(0);
+      if (has) dg = Fi.diag[c];
+      with_coefs(Fi, [&](auto Tx, auto Ty, auto Tz) {
+        if (xm) t0 = Tx[cm];
+        if (xp) t1 = Tx[c];
+        if (ym) t2 = Ty[c - sy];
+        if (yp) t3 = Ty[c];
+        if (zm) t4 = Tz[c - sz];
+        if (zp) t5 = Tz[c];
+      });
+      if (!waited) {
+        MDBS_PDL_WAIT();
+        waited = true;
+      }
+      R r = R(0);
+      if (has) {
+        R x0 = R(0), x1 = R(0), x2 = R(0), x3 = R(0), x4 = R(0), x5 = R(0);
+        const R b = Fi.b[c], xc = x[c];
+        if (xm) x0 = x[cm];
+        if (xp) x1 = x[cp];
+        if (ym) x2 = x[c - sy];
+        if (yp) x3 = x[c + sy];
+        if (zm) x4 = x[c - sz];
+        if (zp) x5 = x[c + sz];
+        R v = R(0);  // resid_cell's chain
+        if (xm) v = fma_r(t0, x0, v);
+        if (xp) v = fma_r(t1, x1, v);
+        if (ym) v = fma_r(t2, x2, v);
+        if (yp) v = fma_r(t3, x3, v);
+        if (zm) v = fma_r(t4, x4, v);
+        if (zp) v = fma_r(t5, x5, v);
+        r = b - (mul_r(dg, xc) - v);
+      }
+      s_res[q][g][t] = r;
     }
+    __syncthreads();
+    if (g == 0 && in) {
+      R s = R(0);
+      for (int p = 0; p < 4; p++)
+        for (int q = 0; q < reps; q++) s += s_res[q][p][t];  // a missing child adds zero
+      Co.b[ci] = s;
+      if (fold && !((Q[0] + Q[1] + Q[2]) & 1)) Co.x[ci] = s * Co.dinv[ci];
+    }
+    __syncthreads();  // s_res is reused
   }
 }
 
@@ -1032,6 +1211,9 @@ __global__ void k_coarse_inverse(const CgDom* __restrict__ CG) {
   }
 }
 
+// ------------------------------------------------------------------ small grids in a cluster
+#include "cluster_solve.cuh"
+
 // ------------------------------------------------------------------ tail V-cycle
 // The small levels (and the coarsest solve) of a V-cycle in one CTA, or in one
 // thread-block cluster of up to 8 CTAs, per domain: the same per-cell arithmetic,
@@ -1105,8 +1287,7 @@ __device__ void tail_restrict(const Level<R>& Fi, const Level<R>& Co, const Tail
           if (mask && ((x + y + z) & 1)) continue;  // as b_resid_restrict
           const int q[3] = {x, y, z};
           const long long c = lpos(Fi.n, x, y, z);
-          const R ax = Fi.diag[c] * Fi.x[c] - neighbour_sum(Fi, Fi.x, q, c);
-          s += Fi.b[c] - ax;
+          s += resid_cell(Fi, Fi.x, Fi.b, q, c);
         }
     Co.b[ci] = s;
   }
@@ -1162,13 +1343,8 @@ __device__ void tail_body(const CgDom& G, int nu1, int nu2, int cs, int smem, co
   }
   const Level<R>& C = lv[nlev - 1];
   if (cs == 0) {
-    const R* cinv = coarse_inverse_of<R>(G);
-    const int n = (int)C.cells;
-    for (int i = (int)tp.first; i < n; i += (int)tp.step) {
-      R v = R(0);
-      for (int j = 0; j < n; j++) v += cinv[i * n + j] * C.b[j];
-      C.x[i] = v;
-    }
+    if (tp.first < blockDim.x)  // one CTA of a cluster
+      coarse_solve(coarse_inverse_of<R>(G), C.b, C.x, (int)C.cells, threadIdx.x, blockDim.x);
     tail_barrier(tp);
   }
   for (int it = 0; it < cs; it++) tail_pair(C, 0, it == 0, tp);
@@ -1399,24 +1575,91 @@ __device__ __forceinline__ double apply_A0(const Fld& F, const Prm& P, const dou
   double v = F.diag[c] * p[nc];
   unsigned o = 1;
   for (int d = 0; d < 3; d++) {
-    if (q[d] > 0) v -= F.T[d][lo_pos(P.n, q, c, d)] * p[nc - o];
-    if (q[d] + 1 < P.n[d]) v -= F.T[d][c] * p[nc + o];
+    if (q[d] > 0) v = fma(-F.T[d][lo_pos(P.n, q, c, d)], p[nc - o], v);
+    if (q[d] + 1 < P.n[d]) v = fma(-F.T[d][c], p[nc + o], v);
     o *= (unsigned)P.n[d];
   }
   return v;
 }
 
-// r = b - A p; one partial of r.r and b.b per block
-template <int REP>
+// The CG vector kernels, in three forms with the same sums.
+//
+// A batch: a work item is one partial sum of a domain (kRepBig rows of kBlock cells), the
+// domains' views come from a table; k_finalize adds the partial sums up.
+//
+// A single domain: its view is passed by value (the pointers come from the constant bank,
+// and a loop of its own needs no test of a flag).  A large one works as a batch does.  One
+// of at most kMidItems sums would occupy as few SMs (61 x 47 x 37 cells are 52 sums): its
+// vector kernels take one row a CTA and form no sum; k_sum_final then runs the sums' chains
+// over the vectors (in L2), and its last block adds them up, in the place of k_finalize.
+// (That block, a step of 23 iterations: 2.38 ms; the rows of a sum dealt out to a cluster of 8
+// CTAs that send their factors to one of them: 2.72 ms.  Above kMidItems the arrivals cost
+// more than the launch saves.)
+constexpr int kMidItems = 256;  // a block of kBlock threads then folds a partial sum a thread
+enum { kBatch = 0, kPlain = 1, kLarge = kRepBig };
+
+// One block's loop over its items: V the domain, lb the index of the partial sum, kRows
+// rows from cell c0 (+ the thread) on.
+#define CG_ITEMS(ITEMS, BLK, REV)                                                                \
+  constexpr int kRows = FORM == kPlain ? 1 : kRepBig;                                            \
+  for (int i_ = blockIdx.x; i_ < (ITEMS); i_ += gridDim.x) {                                     \
+    const int b_ = (REV) ? (ITEMS) - 1 - i_ : i_;                                                \
+    const int dm = FORM != kBatch ? 0 : work_domain((BLK), b_);                                  \
+    const int lb = FORM != kBatch ? b_ : b_ - (BLK).blk[dm];                                     \
+    const CgVec& V = FORM != kBatch ? one : table[dm];                                           \
+    const unsigned c0 = (unsigned)lb * (unsigned)kRows * kBlock + threadIdx.x;
+#define CG_ACTIVE() (FORM != kBatch || V.scal[kCond] != 0.0)
+
+__device__ __forceinline__ void cg_sum(double s, double* out) {
+  s = block_sum(s);
+  if (threadIdx.x == 0) *out = s;
+}
+
+// v_c = (A x)_c at storage position c, x in the storage order given by at(i, j, k, position);
+// the neighbours in the order x-, x+, y-, y+, z-, z+
+__device__ __forceinline__ double apply_row(const CgVec& V, const double* __restrict__ x, unsigned c, double xc) {
+  const unsigned n0 = (unsigned)V.n[0], n1 = (unsigned)V.n[1], n2 = (unsigned)V.n[2], he = (n0 + 1) >> 1;
+  const unsigned row = fastdiv(c, V.dn0), px = c - row * n0;
+  const unsigned k = fastdiv(row, V.dn1), j = row - k * n1;
+  const bool odd = px >= he;
+  const unsigned h = odd ? px - he : px, rb = row * n0;
+  // positions of i - 1 and i + 1: the other parity's run
+  const unsigned cm = odd ? rb + h : rb + he + h - 1, cp = odd ? rb + h + 1 : rb + he + h;
+  const bool xm = odd || h > 0, xp = 2 * h + (odd ? 2u : 1u) < n0;
+  const bool ym = j > 0, yp = j + 1 < n1, zm = k > 0, zp = k + 1 < n2;
+  const unsigned sy = n0, sz = n0 * n1;
+  const double* __restrict__ Tx = V.T[0];
+  const double* __restrict__ Ty = V.T[1];
+  const double* __restrict__ Tz = V.T[2];
+  const double dg = V.diag[c];
+  const double t0 = xm ? Tx[cm] : 0.0, t1 = xp ? Tx[c] : 0.0, t2 = ym ? Ty[c - sy] : 0.0, t3 = yp ? Ty[c] : 0.0,
+               t4 = zm ? Tz[c - sz] : 0.0, t5 = zp ? Tz[c] : 0.0;
+  const double d0 = xm ? x[cm] : 0.0, d1 = xp ? x[cp] : 0.0, d2 = ym ? x[c - sy] : 0.0, d3 = yp ? x[c + sy] : 0.0,
+               d4 = zm ? x[c - sz] : 0.0, d5 = zp ? x[c + sz] : 0.0;
+  double v = dg * xc;
+  v = fma(-t0, d0, v);
+  v = fma(-t1, d1, v);
+  if (n1 > 1) {
+    v = fma(-t2, d2, v);
+    v = fma(-t3, d3, v);
+  }
+  if (n2 > 1) {
+    v = fma(-t4, d4, v);
+    v = fma(-t5, d5, v);
+  }
+  return v;
+}
+
+// r = b - A p; one partial of r.r and b.b per item (p is in natural order)
 __global__ void k_resid0(const StepDom* __restrict__ D, const CgDom* __restrict__ C, Work w, int narrow) {
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK(w)
     const StepDom& S = D[dm];
     const CgDom& G = C[dm];
     double rr = 0.0, bb = 0.0;
-    #pragma unroll
-    for (int r = 0; r < REP; r++) {
-      const long long c = ((long long)lb * REP + r) * blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < kRepBig; r++) {
+      const long long c = ((long long)lb * kRepBig + r) * blockDim.x + threadIdx.x;
       if (c < S.P.cells) {
         int q[3];
         decode_pos(S.P, c, q[0], q[1], q[2]);
@@ -1424,8 +1667,8 @@ __global__ void k_resid0(const StepDom* __restrict__ D, const CgDom* __restrict_
         const double rc = bc - apply_A0(S.F, S.P, S.F.p, (unsigned)c, q);
         G.r[c] = rc;
         if (narrow) G.lf[0].b[c] = (float)rc;  // the first FP32 V-cycle's right-hand side
-        rr += rc * rc;
-        bb += bc * bc;
+        rr = fma(rc, rc, rr);
+        bb = fma(bc, bc, bb);
       }
     }
     rr = block_sum(rr);
@@ -1436,197 +1679,240 @@ __global__ void k_resid0(const StepDom* __restrict__ D, const CgDom* __restrict_
 }
 
 // q = A d; partial d.q
-template <int REP>
-__global__ void k_spmv_dot(const StepDom* __restrict__ D, const CgDom* __restrict__ C, Work w, int rev) {
-  MDBS_DEPENDENT_ENTRY();
-  FOR_WORK_DIR(w, rev)
-    const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
-    const StepDom& S = D[dm];
+template <int FORM>
+__global__ void __launch_bounds__(kBlock, 4)
+    k_spmv_dot(const __grid_constant__ CgVec one, const CgVec* __restrict__ table, Work w, int items, int rev) {
+  MDBS_PDL_TRIGGER();
+  MDBS_PDL_WAIT();
+  CG_ITEMS(items, w, rev)
+    if (!CG_ACTIVE()) continue;
     double s = 0.0;
-    const int n0 = S.P.n[0], n1 = S.P.n[1], n2 = S.P.n[2];
-    const long long n = S.P.cells, sy = n0, sz = (long long)n0 * n1;
-    const double* __restrict__ dv = G.dv;
-    double* __restrict__ qv = G.q;
-    const double* __restrict__ dg = S.F.diag;
-    const double* __restrict__ Tx = S.F.T[0];
-    const double* __restrict__ Ty = S.F.T[1];
-    const double* __restrict__ Tz = S.F.T[2];
-    #pragma unroll 1
-    for (int r = 0; r < REP; r++) {
-      const long long c = ((long long)lb * REP + r) * blockDim.x + threadIdx.x;
-      if (c < n) {
-        int i, j, k;
-        decode_pos(S.P, c, i, j, k);
-        const unsigned rb = (unsigned)n0 * ((unsigned)j + (unsigned)n1 * (unsigned)k), he = (unsigned)(n0 + 1) >> 1;
-        const unsigned cm = rb + xs_px(he, i - 1), cp = rb + xs_px(he, i + 1);
-        const double dc = dv[c];
-        double v = dg[c] * dc;
-        if (i > 0) v -= Tx[cm] * dv[cm];
-        if (i + 1 < n0) v -= Tx[c] * dv[cp];
-        if (j > 0) v -= Ty[c - sy] * dv[c - sy];
-        if (j + 1 < n1) v -= Ty[c] * dv[c + sy];
-        if (k > 0) v -= Tz[c - sz] * dv[c - sz];
-        if (k + 1 < n2) v -= Tz[c] * dv[c + sz];
-        qv[c] = v;
-        s += dc * v;
+#pragma unroll 2
+    for (int r = 0; r < kRows; r++) {
+      const unsigned c = c0 + (unsigned)r * kBlock;
+      if (c < V.cells) {
+        const double dc = V.dv[c];
+        const double v = apply_row(V, V.dv, c, dc);
+        V.q[c] = v;
+        s = fma(dc, v, s);
       }
     }
-    s = block_sum(s);
-    if (threadIdx.x == 0) G.partials[lb] = s;
+    if (FORM != kPlain) cg_sum(s, V.partials + lb);
   }
 }
 
 // p += alpha d; r -= alpha q; partial r.r
-template <int REP>
-__global__ void k_update_xr(const StepDom* __restrict__ D, const CgDom* __restrict__ C, Work w, int rev, int narrow) {
-  MDBS_DEPENDENT_ENTRY();
-  FOR_WORK_DIR(w, rev)
-    const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
-    const StepDom& S = D[dm];
-    const double al = G.scal[kAlpha];
+template <int FORM>
+__global__ void k_update_xr(const __grid_constant__ CgVec one, const CgVec* __restrict__ table, Work w, int items,
+                            int rev, int narrow) {
+  MDBS_PDL_TRIGGER();
+  MDBS_PDL_WAIT();
+  CG_ITEMS(items, w, rev)
+    if (!CG_ACTIVE()) continue;
+    const double al = V.scal[kAlpha];
+    const unsigned n = V.cells, n0 = (unsigned)V.n[0], he = (n0 + 1) >> 1;
+    double* __restrict__ p = V.p;
+    double* __restrict__ rv = V.r;
+    const double* __restrict__ dv = V.dv;
+    const double* __restrict__ qv = V.q;
     double s = 0.0;
-    const long long n = S.P.cells;
-    const unsigned n0 = (unsigned)S.P.n[0], he = (n0 + 1) >> 1;
-    double* __restrict__ p = S.F.p;
-    double* __restrict__ rv = G.r;
-    const double* __restrict__ dv = G.dv;
-    const double* __restrict__ qv = G.q;
-    #pragma unroll
-    for (int r = 0; r < REP; r++) {
-      const long long c = ((long long)lb * REP + r) * blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      const unsigned c = c0 + (unsigned)r * kBlock;
       if (c < n) {
         // p is in natural order: the cell at x-split position c
-        const unsigned row = fastdiv((unsigned)c, S.P.dn0), x = (unsigned)c - row * n0;
-        p[row * n0 + (x < he ? 2 * x : 2 * (x - he) + 1)] += al * dv[c];
-        const double rc = rv[c] - al * qv[c];
+        const unsigned row = fastdiv(c, V.dn0), x = c - row * n0;
+        double* const pc = p + (row * n0 + (x < he ? 2 * x : 2 * (x - he) + 1));
+        *pc = fma(al, dv[c], *pc);
+        const double rc = fma(-al, qv[c], rv[c]);
         rv[c] = rc;
-        if (narrow) G.lf[0].b[c] = (float)rc;  // the next FP32 V-cycle's right-hand side
-        s += rc * rc;
+        if (narrow) V.bf[c] = (float)rc;  // the next FP32 V-cycle's right-hand side
+        s = fma(rc, rc, s);
       }
     }
-    s = block_sum(s);
-    if (threadIdx.x == 0) G.partials[lb] = s;
+    if (FORM != kPlain) cg_sum(s, V.partials + lb);
   }
 }
 
-// partial r.z and (flexible) z.q
-template <int REP>
-__global__ void k_dots_rz(const StepDom* __restrict__ D, const CgDom* __restrict__ C, Work w, int with_zq, int rev) {
-  MDBS_DEPENDENT_ENTRY();
-  FOR_WORK_DIR(w, rev)
-    const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
+// partial r.z and (FLEX) z.q; in flexible CG z is the FP32 V-cycle's result, widened here
+// (no separate pass)
+template <int FORM, bool FLEX>
+__global__ void k_dots_rz(const __grid_constant__ CgVec one, const CgVec* __restrict__ table, Work w, int items,
+                          int rev) {
+  MDBS_PDL_TRIGGER();
+  MDBS_PDL_WAIT();
+  CG_ITEMS(items, w, rev)
+    if (!CG_ACTIVE()) continue;
+    const unsigned n = V.cells;
+    const double* __restrict__ rv = V.r;
+    double* __restrict__ z = V.z;
+    const double* __restrict__ qv = V.q;
+    const float* __restrict__ zf = V.xf;
     double rz = 0.0, zq = 0.0;
-    const long long n = D[dm].P.cells;
-    const double* __restrict__ rv = G.r;
-    double* __restrict__ z = G.z;
-    const double* __restrict__ qv = G.q;
-    const float* __restrict__ zf = G.lf[0].x;
-    #pragma unroll
-    for (int r = 0; r < REP; r++) {
-      const long long c = ((long long)lb * REP + r) * blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      const unsigned c = c0 + (unsigned)r * kBlock;
       if (c < n) {
-        // flexible CG: z is the FP32 V-cycle's result, widened here (no separate pass)
         double zc;
-        if (with_zq) {
+        if (FLEX) {
           zc = (double)zf[c];
           z[c] = zc;
         } else {
           zc = z[c];
         }
-        rz += rv[c] * zc;
-        if (with_zq) zq += zc * qv[c];
+        rz = fma(rv[c], zc, rz);
+        if (FLEX) zq = fma(zc, qv[c], zq);
       }
     }
-    rz = block_sum(rz);
-    if (threadIdx.x == 0) G.partials[lb] = rz;
-    if (with_zq) {
-      zq = block_sum(zq);
-      if (threadIdx.x == 0) G.partials[G.pcap + lb] = zq;
-    }
+    cg_sum(rz, V.partials + lb);
+    if (FLEX) cg_sum(zq, V.partials + V.pcap + lb);
   }
 }
 
 // d = z + beta d; the first iteration (counter 0) takes d = z
-template <int REP>
-__global__ void k_update_d(const StepDom* __restrict__ D, const CgDom* __restrict__ C, Work w, int flexible, int rev) {
-  MDBS_DEPENDENT_ENTRY();
-  FOR_WORK_DIR(w, rev)
-    const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
-    const double* scal = G.scal;
-    const bool first = scal[kIt] == 0.0;
-    double be = 0.0;
-    if (!first) be = flexible ? -scal[kAlpha] * scal[kZQ] / scal[kRZold] : scal[kRZ] / scal[kRZold];
-    const long long n = D[dm].P.cells;
-    const double* __restrict__ z = G.z;
-    double* __restrict__ dv = G.dv;
-    #pragma unroll
-    for (int r = 0; r < REP; r++) {
-      const long long c = ((long long)lb * REP + r) * blockDim.x + threadIdx.x;
-      if (c < n) dv[c] = first ? z[c] : z[c] + be * dv[c];
+template <int FORM>
+__global__ void k_update_d(const __grid_constant__ CgVec one, const CgVec* __restrict__ table, Work w, int items,
+                           int rev) {
+  MDBS_PDL_TRIGGER();
+  MDBS_PDL_WAIT();
+  CG_ITEMS(items, w, rev)
+    if (!CG_ACTIVE()) continue;
+    const bool first = V.scal[kIt] == 0.0;
+    const double be = V.scal[kBeta];
+    const unsigned n = V.cells;
+    const double* __restrict__ z = V.z;
+    double* __restrict__ dv = V.dv;
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      const unsigned c = c0 + (unsigned)r * kBlock;
+      if (c < n) dv[c] = first ? z[c] : fma(be, dv[c], z[c]);
     }
   }
 }
 
-// Scalar finalizers, one block per domain, fixed summation order.  The loop
-// condition "not converged, below max_it, finite" goes to scal[kCond].
+// The CG scalars after the sums a (and b) of a mode (one thread):
 // mode 0: rr, bb after the initial residual; iteration counter = 0
 // mode 1: dq, alpha = rz / dq
 // mode 2: rr after the update; counter += 1
-// mode 3: rz_old = rz; rz (and zq when two channels)
-__global__ void k_finalize(const CgDom* __restrict__ C, Work w, int mode, int two, double tol, int max_it) {
-  MDBS_DEPENDENT_ENTRY();
-  const CgDom& G = C[blockIdx.x];
-  double* scal = G.scal;
-  if (mode != 0 && scal[kCond] == 0.0) return;
-  const int nb = w.blk[blockIdx.x + 1] - w.blk[blockIdx.x];
-  double a = 0.0, b = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-    a += G.partials[i];
-    if (two) b += G.partials[G.pcap + i];
-  }
-  a = block_sum(a);
-  if (two) b = block_sum(b);
-  if (threadIdx.x != 0) return;
+// mode 3: rz and (two sums) zq; beta of the next direction, formed here once: a division in
+//         every warp of k_update_d held the FP64 pipe for 1600 cycles each
+// The loop condition "not converged, below max_it, finite" goes to scal[kCond].
+__device__ __forceinline__ void cg_scalars(double* scal, int mode, int two, double a, double b, double tol, int max_it) {
   if (mode == 1) {
     scal[kDQ] = a;
     scal[kAlpha] = scal[kRZ] / a;
-    return;
-  }
-  if (mode == 3) {
-    scal[kRZold] = scal[kRZ];
+  } else if (mode == 3) {
+    const double old = scal[kRZ];
+    scal[kBeta] = two ? -scal[kAlpha] * b / old : a / old;
     scal[kRZ] = a;
-    scal[kZQ] = two ? b : 0.0;
-    return;
-  }
-  double it;
-  if (mode == 0) {
-    scal[kRR] = a;
-    scal[kBB] = b;
-    it = 0.0;
   } else {
+    const double it = mode == 0 ? 0.0 : scal[kIt] + 1.0;
+    const double bb = mode == 0 ? b : scal[kBB];
     scal[kRR] = a;
-    it = scal[kIt] + 1.0;
+    scal[kBB] = bb;
+    scal[kIt] = it;
+    const bool done = bb == 0.0 || sqrt(a) <= tol * sqrt(bb) || it >= (double)max_it || !(a == a);
+    scal[kCond] = done ? 0.0 : 1.0;
   }
-  scal[kIt] = it;
-  const double bb = scal[kBB];
-  const bool done = bb == 0.0 || sqrt(a) <= tol * sqrt(bb) || it >= (double)max_it || !(a == a);
-  scal[kCond] = done ? 0.0 : 1.0;
 }
 
-// OR of the domains' conditions: the WHILE node's condition (captured graph) and a flag
-// the host reads (eager loop)
-__global__ void k_any(const CgDom* __restrict__ C, int ndom, int* flag, cudaGraphConditionalHandle handle,
-                      int use_handle) {
+// Scalar finalizers, one block per domain, fixed summation order (cg_scalars' modes).
+// Modes 0 and 2 also decide whether any domain goes on: the block that arrives last ORs the
+// conditions into *flag (the eager loop reads it) and the WHILE node's condition.
+__global__ void k_finalize(const CgDom* __restrict__ C, Work w, int mode, int two, double tol, int max_it, int* flag,
+                           cudaGraphConditionalHandle handle, int use_handle) {
   MDBS_DEPENDENT_ENTRY();
+  const CgDom& G = C[blockIdx.x];
+  double* scal = G.scal;
+  const int nb = w.blk[blockIdx.x + 1] - w.blk[blockIdx.x];  // 0: solved by the cluster kernel
+  if (nb > 0 && (mode == 0 || scal[kCond] != 0.0)) {
+    double a = 0.0, b = 0.0;
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+      a += G.partials[i];
+      if (two) b += G.partials[G.pcap + i];
+    }
+    a = block_sum(a);
+    if (two) b = block_sum(b);
+    if (threadIdx.x == 0) cg_scalars(scal, mode, two, a, b, tol, max_it);
+  }
+  if (mode == 1 || mode == 3) return;
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = gridDim.x == 1 || atomicAdd(flag + 1, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
   int any = 0;
-  for (int d = threadIdx.x; d < ndom; d += blockDim.x) any |= C[d].scal[kCond] != 0.0;
+  for (int d = threadIdx.x; d < (int)gridDim.x; d += blockDim.x) any |= __ldcg(C[d].scal + kCond) != 0.0;
   any = __syncthreads_or(any);
   if (threadIdx.x == 0) {
-    *flag = any;
+    flag[0] = any;
+    flag[1] = 0;
+    if (use_handle) cudaGraphSetConditional(handle, any ? 1u : 0u);
+  }
+}
+
+// The sums of one mode of a single domain of at most kMidItems partial sums, one a block,
+// and, in the block that arrives last, their total in k_finalize's order and the scalars.
+// mode 1: d.q; mode 2: r.r; mode 3: r.z and (FLEX) z.q, z widened from the FP32 V-cycle.
+template <int MODE, bool FLEX>
+__global__ void __launch_bounds__(kBlock)
+    k_sum_final(const __grid_constant__ CgVec V, double tol, int max_it, int* flag, cudaGraphConditionalHandle handle,
+                int use_handle) {
+  MDBS_PDL_TRIGGER();
+  MDBS_PDL_WAIT();
+  constexpr bool kTwo = MODE == 3 && FLEX;
+  const int lb = blockIdx.x;
+  const unsigned n = V.cells, c0 = (unsigned)lb * (kRepBig * kBlock) + threadIdx.x;
+  const double* __restrict__ rv = V.r;
+  double* __restrict__ z = V.z;
+  const double* __restrict__ dv = V.dv;
+  const double* __restrict__ qv = V.q;
+  const float* __restrict__ zf = V.xf;
+  double a = 0.0, b = 0.0;
+#pragma unroll
+  for (int r = 0; r < kRepBig; r++) {
+    const unsigned c = c0 + (unsigned)r * kBlock;
+    if (c < n) {
+      if (MODE == 1) {
+        a = fma(dv[c], qv[c], a);
+      } else if (MODE == 2) {
+        const double rc = rv[c];
+        a = fma(rc, rc, a);
+      } else {
+        double zc;
+        if (FLEX) {
+          zc = (double)zf[c];
+          z[c] = zc;
+        } else {
+          zc = z[c];
+        }
+        a = fma(rv[c], zc, a);
+        if (FLEX) b = fma(zc, qv[c], b);
+      }
+    }
+  }
+  cg_sum(a, V.partials + lb);
+  if (kTwo) cg_sum(b, V.partials + V.pcap + lb);
+  __shared__ int s_last;
+  __syncthreads();  // the sums are written (by thread 0 or lane 0 of the first warp)
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(flag + 1, 1) == (int)gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last) return;
+  const int i = threadIdx.x;
+  a = block_sum(i < (int)gridDim.x ? __ldcg(V.partials + i) : 0.0);
+  if (kTwo) b = block_sum(i < (int)gridDim.x ? __ldcg(V.partials + V.pcap + i) : 0.0);
+  if (threadIdx.x != 0) return;
+  cg_scalars(V.scal, MODE, kTwo, a, b, tol, max_it);
+  flag[1] = 0;
+  if (MODE == 2) {
+    const int any = V.scal[kCond] != 0.0;
+    flag[0] = any;
     if (use_handle) cudaGraphSetConditional(handle, any ? 1u : 0u);
   }
 }
@@ -1636,8 +1922,8 @@ __global__ void k_zero_if_b0(const StepDom* __restrict__ D, const CgDom* __restr
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK(w)
     if (C[dm].scal[kBB] != 0.0) continue;
-    for (int r = 0; r < w.rep; r++) {
-      const long long c = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
+    for (int r = 0; r < kRepBig; r++) {
+      const long long c = ((long long)lb * kRepBig + r) * blockDim.x + threadIdx.x;
       if (c < D[dm].P.cells) D[dm].F.p[c] = 0.0;
     }
   }
@@ -1709,6 +1995,14 @@ cudaError_t sweep_kernel_setup() {
     e = cudaFuncSetAttribute(k_coarse_coop<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_coarse_coop<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMax);
+  const void* cl[] = {(const void*)k_tail_cluster<double>, (const void*)k_tail_cluster<float>,
+                      (const void*)k_cg_cluster<double, 1>, (const void*)k_cg_cluster<double, 2>,
+                      (const void*)k_cg_cluster<double, 4>, (const void*)k_cg_cluster<float, 1>,
+                      (const void*)k_cg_cluster<float, 2>, (const void*)k_cg_cluster<float, 4>};
+  for (const void* k : cl) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
   return e;
 }
 
@@ -1717,6 +2011,58 @@ cudaError_t sweep_kernel_setup() {
 static size_t tail_smem_bytes(const BatchPlan& B, size_t word, int ctas) {
   const size_t bytes = (size_t)B.tail_words * word;
   return ctas == 1 && bytes <= kTailSmemMax ? bytes : 0;
+}
+
+// Which domains the cluster kernels take and with what launch shape.  Small domains (every
+// level in the tail, at most kClCells cells) run their whole CG solve in a cluster; the
+// others' tails run in one when every tail starts at a level of at most kClCells cells.
+// More CTAs share a level's FP64 work; with many domains the GPU is full without.
+cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas, int sms, BatchPlan* B) {
+  auto ctas_for = [](long long cells, int per) {
+    int c = 1;
+    while ((long long)c * per < cells) c *= 2;
+    return c;
+  };
+  auto bytes = [&](int d, int first, int ctas, int rows) {
+    // as without pre-smoothing, when the restriction sums all children
+    return flexible ? cl_bytes<float>(cg[d].lf, first, cg[d].nlev, ctas, rows, 0)
+                    : cl_bytes<double>(cg[d].ld, first, cg[d].nlev, ctas, rows, 0);
+  };
+  bool tails = B->n_big > 0;
+  long long most_small = 1, most = 1;
+  for (int d = 0; d < ndom; d++) {
+    if (cg[d].small) {
+      if (cg[d].ld[0].cells > most_small) most_small = cg[d].ld[0].cells;
+    } else {
+      const long long n = cg[d].ld[cg[d].first].cells;
+      if (cg[d].first == 0 || n > kClCells) tails = false;
+      if (n > most) most = n;
+    }
+  }
+  // one reduction row a CTA while every CTA then has an SM of its own, else more
+  auto small_for = [&](int rows) {
+    if (most_small <= kClRow * rows) return 1;
+    return (int)((most_small + kClSum - 1) / kClSum) * (kRepBig / rows);
+  };
+  B->small_rows = 1;
+  while (B->small_rows < kClRowsMax && B->n_small * small_for(B->small_rows) > sms) B->small_rows *= 2;
+  for (;; B->small_rows /= 2) {
+    B->small_ctas = small_for(B->small_rows);
+    B->small_smem = 0;
+    for (int d = 0; d < ndom; d++)
+      if (cg[d].small) B->small_smem = std::max(B->small_smem, bytes(d, 0, B->small_ctas, B->small_rows));
+    if (B->small_smem <= kClSmemMax || B->small_rows == 1) break;
+  }
+  int ctas = 0;
+  if (tails) {
+    ctas = tail_ctas > 1 ? tail_ctas : ctas_for(most, kClRow);
+    while (tail_ctas == 1 && ctas > 4 && ctas * B->n_big > sms) ctas /= 2;
+  }
+  for (int d = 0; d < ndom; d++)
+    if (ctas && !cg[d].small) B->cl_tail_smem = std::max(B->cl_tail_smem, bytes(d, cg[d].first, ctas, 0));
+  if (B->cl_tail_smem > kClSmemMax) ctas = 0;
+  B->cl_tail_ctas = ctas;
+  return B->small_smem <= kClSmemMax ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
 cudaError_t coop_grid_size(int flexible, long long tail_words, int* grid) {
@@ -1789,7 +2135,7 @@ static size_t solver_layout(const int n[3], int precision, PressureSolver* ps, c
     return p;
   };
   const long long n0 = (long long)n[0] * n[1] * n[2];
-  const long long pcap = (n0 + kBlock * kRepBig - 1) / (kBlock * kRepBig);
+  const long long pcap = cg_items(n0);
   double* r = (double*)take(n0 * 8);
   double* z = (double*)take(n0 * 8);
   double* z2 = (double*)take(n0 * 8);
@@ -1968,6 +2314,7 @@ void pressure_view(const PressureSolver* ps, const Fld& F, int tail_cells, CgDom
   int first = ps->nlev - 1;
   while (first > 0 && ps->ld[first - 1].cells <= tail_cells) first--;
   G.first = first;
+  G.small = first == 0 && ps->ld[0].cells <= kClCells;
   G.r = ps->r;
   G.z = ps->z;
   G.dv = ps->dv;
@@ -2023,6 +2370,17 @@ struct Dirs {
   }
 };
 
+// levels l and l + 1 of the plan's only domain (a batch reads its table instead)
+template <typename R>
+static LvPair<R> level_pair(const BatchPlan& B, int l) {
+  LvPair<R> p{};
+  if (!B.one_cg) return p;
+  const Level<R>* L = std::is_same<R, float>::value ? (const Level<R>*)B.one_cg->lf : (const Level<R>*)B.one_cg->ld;
+  p.fine = L[l];
+  if (l + 1 < B.one_cg->nlev) p.coarse = L[l + 1];
+  return p;
+}
+
 // pro: the half sweep applies the prolongation from level l + 1 to the neighbours
 // it reads (the first post-smoothing half sweep; no separate prolongation launch)
 template <typename R, bool PRO>
@@ -2040,7 +2398,11 @@ static void smooth_half_t(const BatchPlan& B, int l, int col, int zero, Dirs& D,
     case 8: MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_smooth<R, 8, PRO>), B.cg, w, l, col, zero, rev); break;
     case 4: MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_smooth<R, 4, PRO>), B.cg, w, l, col, zero, rev); break;
     case 2: MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_smooth<R, 2, PRO>), B.cg, w, l, col, zero, rev); break;
-    default: MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_smooth<R, 1, PRO>), B.cg, w, l, col, zero, rev); break;
+    default:
+      if (B.one_cg)
+        MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_sweep<R, PRO>), level_pair<R>(B, l), w.total, col, zero, rev);
+      else
+        MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_smooth<R, 1, PRO>), B.cg, w, l, col, zero, rev);
   }
 }
 
@@ -2074,6 +2436,26 @@ static void sweep(const BatchPlan& B, int l, int first_col, bool zero, int src, 
   }
 }
 
+// ndom clusters of ctas CTAs
+template <typename K, typename... A>
+static cudaError_t launch_cluster(K kernel, int ndom, int ctas, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ndom * ctas);
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = ctas;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = ctas > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Symmetric V-cycle of every active domain: level 0 receives M r.  Levels that
 // precede a domain's tail start run as batched launches; the rest of each
 // domain's cycle runs in its own CTA of the tail kernel.  With fused sweeps a
@@ -2101,8 +2483,15 @@ static void vcycle(const BatchPlan& B, int nu1, int nu2, int cs, Dirs& D, cudaSt
       else
         sweep<R>(B, l, 0, it == 0, cur(it), D, s);
     }
-    MDBS_LAUNCH(l == 0 ? K_RESTRICT0 : K_RESTRICTC, grid_of(B, B.lcoarse[l]), kBlock, s, k_resid_restrict<R>, B.cg,
-                B.lcoarse[l], l, D.next(l), cur(nu1), nu1 > 0 ? 1 : 0, (fold && l + 1 < batched_end) ? 1 : 0);
+    const LvPair<R> one = level_pair<R>(B, l);
+    const int id = l == 0 ? K_RESTRICT0 : K_RESTRICTC, rev = D.next(l);
+    const int mask = nu1 > 0 ? 1 : 0, store = (fold && l + 1 < batched_end) ? 1 : 0;
+    const Work& wr = B.lrest[l];
+    if (B.one_cg)
+      MDBS_LAUNCH(id, grid_of(B, wr), kBlock, s, (k_resid_restrict<R, true>), one, B.cg, wr, l, rev, cur(nu1), mask, store);
+    else
+      MDBS_LAUNCH(id, grid_of(B, wr), kBlock, s, (k_resid_restrict<R, false>), one, B.cg, wr, l, rev, cur(nu1), mask,
+                  store);
   }
   if (coop) {
     const size_t smem = tail_smem_bytes(B, sizeof(R), 1);
@@ -2131,10 +2520,17 @@ static void vcycle(const BatchPlan& B, int nu1, int nu2, int cs, Dirs& D, cudaSt
     if (le != cudaSuccess) set_launch_error(le);
     prof_end(K_COOP, s);
   }
+  if (!coop && B.cl_tail_ctas > 0) {
+    prof_begin(K_TAIL, s);
+    const cudaError_t le = launch_cluster(k_tail_cluster<R>, B.n_big, B.cl_tail_ctas, B.cl_tail_smem, s, B.cg, B.big_idx,
+                                          B.cl_tail_ctas, nu1, nu2, cs);
+    if (le != cudaSuccess) set_launch_error(le);
+    prof_end(K_TAIL, s);
+  }
   const int ctas = B.tail_ctas;
   const size_t tail_bytes = (size_t)B.tail_words * sizeof(R);
   const int tail_smem = ctas == 1 && tail_bytes <= kTailSmemMax ? 1 : 0;
-  if (!coop) {
+  if (!coop && B.cl_tail_ctas == 0) {
     prof_begin(K_TAIL, s);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(B.ndom * ctas);
@@ -2172,6 +2568,28 @@ cudaError_t pressure_solve(const BatchPlan& B, double tol, int max_it, int nu1, 
                            bool capture, cudaStream_t s, cudaStream_t body_stream, double* host_flag,
                            long long* body_launches) {
   const int flexible = B.flexible;  // the hierarchy comes from launch_pressure_matrix
+  if (B.n_small > 0) {
+    prof_begin(K_CG_CLUSTER, s);
+    auto launch = [&](auto kernel) {
+      return launch_cluster(kernel, B.n_small, B.small_ctas, B.small_smem, s, B.sd, B.cg, B.small_idx, B.small_ctas, nu1,
+                            nu2, cs, tol, max_it);
+    };
+    const int rows = B.small_rows;
+    const cudaError_t le = flexible ? (rows == 1   ? launch(k_cg_cluster<float, 1>)
+                                       : rows == 2 ? launch(k_cg_cluster<float, 2>)
+                                                   : launch(k_cg_cluster<float, 4>))
+                                    : (rows == 1   ? launch(k_cg_cluster<double, 1>)
+                                       : rows == 2 ? launch(k_cg_cluster<double, 2>)
+                                                   : launch(k_cg_cluster<double, 4>));
+    if (le != cudaSuccess) set_launch_error(le);
+    prof_end(K_CG_CLUSTER, s);
+  }
+  if (B.n_big == 0) {
+    if (body_launches) *body_launches = 0;
+    MDBS_LAUNCH(K_FINALIZE, B.ndom, 32, s, k_record, B.sd, B.cg, corr, tol);
+    const cudaError_t le = take_launch_error();
+    return le != cudaSuccess ? le : cudaGetLastError();
+  }
   cudaGraphConditionalHandle handle = 0;
   cudaGraph_t graph = nullptr;
   if (capture) {
@@ -2186,12 +2604,12 @@ cudaError_t pressure_solve(const BatchPlan& B, double tol, int max_it, int nu1, 
   }
   const int use = capture ? 1 : 0;
   // initial residual and loop condition
-  MDBS_LAUNCH(K_RESID0, grid_of(B, B.rcells), kBlock, s, (k_resid0<kRepBig>), B.sd, B.cg, B.rcells, flexible);
-  MDBS_LAUNCH(K_FINALIZE, B.ndom, 1024, s, k_finalize, B.cg, B.rcells, 0, 1, tol, max_it);
-  MDBS_LAUNCH(K_FINALIZE, 1, 1024, s, k_any, B.cg, B.ndom, B.any_flag, handle, use);
-  MDBS_LAUNCH(K_ZERO, grid_of(B, B.cells), kBlock, s, k_zero_if_b0, B.sd, B.cg, B.cells);
+  MDBS_LAUNCH(K_RESID0, grid_of(B, B.cgcells), kBlock, s, k_resid0, B.sd, B.cg, B.cgcells, flexible);
+  MDBS_LAUNCH(K_FINALIZE, B.ndom, 1024, s, k_finalize, B.cg, B.cgcells, 0, 1, tol, max_it, B.any_flag, handle, use);
+  MDBS_LAUNCH(K_ZERO, grid_of(B, B.cgcells), kBlock, s, k_zero_if_b0, B.sd, B.cg, B.cgcells);
   // one CG iteration, preconditioner first; the last kernels decide whether to continue
   Dirs D(B.snake);
+  const int grid = grid_of(B, B.cgcells);
   auto body = [&](cudaStream_t bs) {
     if (!flexible) {
       vcycle<double>(B, nu1, nu2, cs, D, bs);
@@ -2200,15 +2618,41 @@ cudaError_t pressure_solve(const BatchPlan& B, double tol, int max_it, int nu1, 
       // widened by the dot products
       vcycle<float>(B, nu1, nu2, cs, D, bs);
     }
-    MDBS_LAUNCH(K_DOTS, grid_of(B, B.rcells), kBlock, bs, (k_dots_rz<kRepBig>), B.sd, B.cg, B.rcells, flexible, D.next(0));
-    MDBS_LAUNCH(K_FINALIZE, B.ndom, 1024, bs, k_finalize, B.cg, B.rcells, 3, flexible, tol, max_it);
-    MDBS_LAUNCH(K_UPDATE_D, grid_of(B, B.rcells), kBlock, bs, (k_update_d<kRepBig>), B.sd, B.cg, B.rcells, flexible, D.next(0));
-    MDBS_LAUNCH(K_SPMV_DOT, grid_of(B, B.rcells), kBlock, bs, (k_spmv_dot<kRepBig>), B.sd, B.cg, B.rcells, D.next(0));
-    MDBS_LAUNCH(K_FINALIZE, B.ndom, 1024, bs, k_finalize, B.cg, B.rcells, 1, 0, tol, max_it);
-    MDBS_LAUNCH(K_UPDATE_XR, grid_of(B, B.rcells), kBlock, bs, (k_update_xr<kRepBig>), B.sd, B.cg, B.rcells, D.next(0),
-                flexible);
-    MDBS_LAUNCH(K_FINALIZE, B.ndom, 1024, bs, k_finalize, B.cg, B.rcells, 2, 0, tol, max_it);
-    MDBS_LAUNCH(K_FINALIZE, 1, 1024, bs, k_any, B.cg, B.ndom, B.any_flag, handle, use);
+    auto finalize = [&](int mode, int two) {
+      MDBS_LAUNCH(K_FINALIZE, B.ndom, 1024, bs, k_finalize, B.cg, B.cgcells, mode, two, tol, max_it, B.any_flag, handle,
+                  use);
+    };
+    const Work& w = B.cgcells;
+    if (B.ndom == 1 && w.total <= kMidItems) {
+      const int rows = (int)((B.one_cv.cells + kBlock - 1) / kBlock);
+      auto sums = [&](int id, auto kernel) {
+        MDBS_LAUNCH(id, w.total, kBlock, bs, kernel, B.one_cv, tol, max_it, B.any_flag, handle, use);
+      };
+      sums(K_DOTS, flexible ? k_sum_final<3, true> : k_sum_final<3, false>);
+      MDBS_LAUNCH(K_UPDATE_D, rows, kBlock, bs, (k_update_d<kPlain>), B.one_cv, B.cv, w, rows, D.next(0));
+      MDBS_LAUNCH(K_SPMV_DOT, rows, kBlock, bs, (k_spmv_dot<kPlain>), B.one_cv, B.cv, w, rows, D.next(0));
+      sums(K_DOTS, k_sum_final<1, false>);
+      MDBS_LAUNCH(K_UPDATE_XR, rows, kBlock, bs, (k_update_xr<kPlain>), B.one_cv, B.cv, w, rows, D.next(0), flexible);
+      sums(K_DOTS, k_sum_final<2, false>);
+      return;
+    }
+    auto vectors = [&](auto form) {
+      constexpr int FORM = decltype(form)::value;
+      if (flexible)
+        MDBS_LAUNCH(K_DOTS, grid, kBlock, bs, (k_dots_rz<FORM, true>), B.one_cv, B.cv, w, w.total, D.next(0));
+      else
+        MDBS_LAUNCH(K_DOTS, grid, kBlock, bs, (k_dots_rz<FORM, false>), B.one_cv, B.cv, w, w.total, D.next(0));
+      finalize(3, flexible);
+      MDBS_LAUNCH(K_UPDATE_D, grid, kBlock, bs, (k_update_d<FORM>), B.one_cv, B.cv, w, w.total, D.next(0));
+      MDBS_LAUNCH(K_SPMV_DOT, grid, kBlock, bs, (k_spmv_dot<FORM>), B.one_cv, B.cv, w, w.total, D.next(0));
+      finalize(1, 0);
+      MDBS_LAUNCH(K_UPDATE_XR, grid, kBlock, bs, (k_update_xr<FORM>), B.one_cv, B.cv, w, w.total, D.next(0), flexible);
+      finalize(2, 0);
+    };
+    if (B.ndom == 1)
+      vectors(std::integral_constant<int, kLarge>{});
+    else
+      vectors(std::integral_constant<int, kBatch>{});
   };
   if (capture) {
     cudaStreamCaptureStatus st;
