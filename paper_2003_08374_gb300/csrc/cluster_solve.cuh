@@ -47,6 +47,7 @@ struct ClLevel {
   int lcol;      // log2 of the columns (of kClRow) a CTA holds of each row; -1: contiguous positions
   int here;      // cells in this CTA
   int red;       // of these, colour 0
+  int most;      // the larger of its counts of the two colours
   int ne;        // neighbours per cell: 2, 4 or 6
   int cap;       // slots the arrays are sized for (stride of coef, nb and ch)
   int nch;       // residuals of the finer level that make up a right-hand side
@@ -161,6 +162,13 @@ __device__ __forceinline__ void sh_st(unsigned a, unsigned v) { asm volatile("st
 __device__ __forceinline__ void sh_st16(unsigned a, unsigned v) {
   asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
 }
+// predicated stores: no branch around them, which costs as much as a phase's loads
+__device__ __forceinline__ void sh_st_if(unsigned a, double v, bool ok) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.shared.f64 [%0], %1;\n}\n" ::"r"(a), "d"(v), "r"((unsigned)ok) : "memory");
+}
+__device__ __forceinline__ void sh_st_if(unsigned a, float v, bool ok) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.shared.f32 [%0], %1;\n}\n" ::"r"(a), "f"(v), "r"((unsigned)ok) : "memory");
+}
 __device__ __forceinline__ void cl_ld(unsigned a, double& v) {
   asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
 }
@@ -189,23 +197,27 @@ __device__ __forceinline__ void cl_wait() {
 // phases of the cluster that is an arrival at the cluster barrier, which the next phase
 // (or whoever reads the result) waits for.
 //
-// The phases are functions of their own, not inlined: a V-cycle runs each of them dozens of
-// times, and with a copy at every call site the instruction fetches took most of a phase's
-// time (a half sweep of 64 cells 640-830 cycles, of which 200-450 are FP64).  They take
-// shared addresses (sm: none needed; lv: a ClLevel), so nothing lives in local memory.
+// Who runs a phase is a template parameter and each phase has one or two call sites, so
+// that everything is inlined.  (As functions of their own they were no faster, and with four
+// rows a CTA, where caller and callee together are short of registers, nvcc 13.0 built a
+// kernel whose results were wrong on one shape, 9 x 20 x 11.)  They take shared addresses
+// (lv: a ClLevel), so nothing lives in local memory.
 enum { kByCluster = 0, kByBlock = 1, kByWarp = 2 };
-__device__ __forceinline__ void cl_begin(int kind) {
-  if (kind == kByCluster)
+template <int KIND>
+__device__ __forceinline__ void cl_begin() {
+  if constexpr (KIND == kByCluster)
     cl_wait();
-  else if (kind == kByBlock)
+  else if constexpr (KIND == kByBlock)
     __syncthreads();
   else
     __syncwarp();
 }
-__device__ __forceinline__ void cl_end(int kind) {
-  if (kind == kByCluster) cl_arrive();
+template <int KIND>
+__device__ __forceinline__ void cl_end() {
+  if constexpr (KIND == kByCluster) cl_arrive();
 }
-__device__ __forceinline__ unsigned cl_step(int kind) { return kind == kByWarp ? 32u : (unsigned)kClThreads; }
+template <int KIND>
+constexpr unsigned kClStep = KIND == kByWarp ? 32u : (unsigned)kClThreads;
 // field of the ClLevel at shared address lv
 #define CL_F(lv, field) sh_ldw((lv) + (unsigned)offsetof(ClLevel, field))
 
@@ -219,12 +231,12 @@ struct Cl {
 
 // One red-black half sweep over this CTA's cells of colour col (zero: the other colour's x
 // is taken as 0).
-template <typename R, int NE>
-__device__ __forceinline__ void cl_half_ne(unsigned lv, int col, int zero, int kind) {
+template <typename R, int KIND, int NE>
+__device__ __forceinline__ void cl_half_ne(unsigned lv, int col, int zero) {
   constexpr unsigned W = sizeof(R);
   const unsigned cap = CL_F(lv, cap), red = CL_F(lv, red), here = CL_F(lv, here);
   const unsigned x = CL_F(lv, x), b = CL_F(lv, b), dinv = CL_F(lv, dinv), cf = CL_F(lv, coef), nb = CL_F(lv, nb);
-  const unsigned last = col ? here : red, step = cl_step(kind);
+  const unsigned last = col ? here : red, step = kClStep<KIND>;
   unsigned e = (col ? red : 0u) + threadIdx.x;
   unsigned a[NE] = {};
   R k[NE] = {}, di = R(0);
@@ -239,7 +251,7 @@ __device__ __forceinline__ void cl_half_ne(unsigned lv, int col, int zero, int k
     }
   };
   if (e < last) fetch();
-  cl_begin(kind);
+  cl_begin<KIND>();
   while (e < last) {
     R v, xn[NE];
     sh_ld(b + e * W, v);
@@ -253,24 +265,24 @@ __device__ __forceinline__ void cl_half_ne(unsigned lv, int col, int zero, int k
     e += step;
     if (e < last) fetch();
   }
-  cl_end(kind);
+  cl_end<KIND>();
 }
-template <typename R>
-__device__ __noinline__ void cl_half(unsigned lv, int col, int zero, int kind) {
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_half(unsigned lv, int col, int zero) {
   const unsigned ne = CL_F(lv, ne);
   if (ne == 6)
-    cl_half_ne<R, 6>(lv, col, zero, kind);
+    cl_half_ne<R, KIND, 6>(lv, col, zero);
   else if (ne == 4)
-    cl_half_ne<R, 4>(lv, col, zero, kind);
+    cl_half_ne<R, KIND, 4>(lv, col, zero);
   else
-    cl_half_ne<R, 2>(lv, col, zero, kind);
+    cl_half_ne<R, KIND, 2>(lv, col, zero);
 }
 
 // residual b - A x of this CTA's cells (mask: colour 0 only), into res
-template <typename R, int NE>
-__device__ __forceinline__ void cl_resid_ne(unsigned lv, int mask, int kind) {
+template <typename R, int KIND, int NE>
+__device__ __forceinline__ void cl_resid_ne(unsigned lv, int mask) {
   constexpr unsigned W = sizeof(R);
-  const unsigned cap = CL_F(lv, cap), last = mask ? CL_F(lv, red) : CL_F(lv, here), step = cl_step(kind);
+  const unsigned cap = CL_F(lv, cap), last = mask ? CL_F(lv, red) : CL_F(lv, here), step = kClStep<KIND>;
   const unsigned x = CL_F(lv, x), b = CL_F(lv, b), dg = CL_F(lv, diag), cf = CL_F(lv, coef), nb = CL_F(lv, nb);
   const unsigned res = CL_F(lv, res), ord = CL_F(lv, ord);
   unsigned e = threadIdx.x, pos = 0;
@@ -286,7 +298,7 @@ __device__ __forceinline__ void cl_resid_ne(unsigned lv, int mask, int kind) {
     }
   };
   if (e < last) fetch();
-  cl_begin(kind);
+  cl_begin<KIND>();
   while (e < last) {
     R xn[NE], xo;
     sh_ld(b + e * W, bv);
@@ -300,53 +312,77 @@ __device__ __forceinline__ void cl_resid_ne(unsigned lv, int mask, int kind) {
     e += step;
     if (e < last) fetch();
   }
-  cl_end(kind);
+  cl_end<KIND>();
 }
-template <typename R>
-__device__ __noinline__ void cl_resid(unsigned lv, int mask, int kind) {
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_resid(unsigned lv, int mask) {
   const unsigned ne = CL_F(lv, ne);
   if (ne == 6)
-    cl_resid_ne<R, 6>(lv, mask, kind);
+    cl_resid_ne<R, KIND, 6>(lv, mask);
   else if (ne == 4)
-    cl_resid_ne<R, 4>(lv, mask, kind);
+    cl_resid_ne<R, KIND, 4>(lv, mask);
   else
-    cl_resid_ne<R, 2>(lv, mask, kind);
+    cl_resid_ne<R, KIND, 2>(lv, mask);
 }
 
 // right-hand side of the level at lv: its children's residuals summed in the order of
-// b_resid_restrict; fold: also its zero-guess colour-0 update
-template <typename R>
-__device__ __noinline__ void cl_gather(unsigned lv, int fold, int kind) {
+// b_resid_restrict; fold: also its zero-guess colour-0 update.  Lanes beyond the cells
+// repeat cell 0 and store nothing; warps beyond them do nothing.
+template <typename R, int KIND, int NCH>
+__device__ __forceinline__ void cl_gather_n(unsigned lv, int fold) {
   constexpr unsigned W = sizeof(R);
-  const unsigned cap = CL_F(lv, cap), here = CL_F(lv, here), red = CL_F(lv, red), nch = CL_F(lv, nch);
-  const unsigned b = CL_F(lv, b), x = CL_F(lv, x), dinv = CL_F(lv, dinv), ch = CL_F(lv, ch), step = cl_step(kind);
-  unsigned e = threadIdx.x;
-  cl_begin(kind);
-  for (; e < here; e += step) {
-    R r[8], di = R(0);
+  const unsigned cap = CL_F(lv, cap), here = CL_F(lv, here), red = CL_F(lv, red);
+  const unsigned b = CL_F(lv, b), x = CL_F(lv, x), dinv = CL_F(lv, dinv), ch = CL_F(lv, ch), step = kClStep<KIND>;
+  const unsigned lane = threadIdx.x & 31u;
+  unsigned a[NCH], e = 0;
+  R di = R(0);
+  bool ok = false;
+  auto fetch = [&](unsigned base) {
+    ok = base + lane < here;
+    e = ok ? base + lane : 0u;
 #pragma unroll
-    for (unsigned q = 0; q < 8; q++)
-      if (q < nch) cl_ld(sh_ldw(ch + (q * cap + e) * 4u), r[q]);
-    if (fold) sh_ld(dinv + e * W, di);
+    for (int q = 0; q < NCH; q++) a[q] = sh_ldw(ch + ((unsigned)q * cap + e) * 4u);
+    sh_ld(dinv + e * W, di);
+  };
+  unsigned base = threadIdx.x - lane;
+  if (base < here) fetch(base);
+  cl_begin<KIND>();
+  while (base < here) {
+    R r[NCH];
+#pragma unroll
+    for (int q = 0; q < NCH; q++) cl_ld(a[q], r[q]);
     R s = R(0);
 #pragma unroll
-    for (unsigned q = 0; q < 8; q++)
-      if (q < nch) s += r[q];
-    sh_st(b + e * W, s);
-    if (fold && e < red) sh_st(x + e * W, s * di);
+    for (int q = 0; q < NCH; q++) s += r[q];
+    sh_st_if(b + e * W, s, ok);
+    if (fold && base < red) sh_st_if(x + e * W, s * di, ok && e < red);
+    base += step;
+    if (base < here) fetch(base);
   }
-  cl_end(kind);
+  cl_end<KIND>();
+}
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_gather(unsigned lv, int fold) {
+  const unsigned n = CL_F(lv, nch);
+  if (n == 1)
+    cl_gather_n<R, KIND, 1>(lv, fold);
+  else if (n == 2)
+    cl_gather_n<R, KIND, 2>(lv, fold);
+  else if (n == 4)
+    cl_gather_n<R, KIND, 4>(lv, fold);
+  else
+    cl_gather_n<R, KIND, 8>(lv, fold);
 }
 
 // x += the parents' x; only colour 0 when a half sweep of colour 1 follows (that sweep
 // reads colour 0 alone and overwrites colour 1)
-template <typename R>
-__device__ __noinline__ void cl_prolong(unsigned lv, int red_only, int kind) {
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_prolong(unsigned lv, int red_only) {
   constexpr unsigned W = sizeof(R);
   const unsigned last = red_only ? CL_F(lv, red) : CL_F(lv, here), x = CL_F(lv, x), par = CL_F(lv, par);
-  const unsigned step = cl_step(kind);
+  const unsigned step = kClStep<KIND>;
   unsigned e = threadIdx.x;
-  cl_begin(kind);
+  cl_begin<KIND>();
   for (; e < last; e += step) {
     R xv, ev;
     const unsigned a = sh_ldw(par + e * 4u);
@@ -354,15 +390,15 @@ __device__ __noinline__ void cl_prolong(unsigned lv, int red_only, int kind) {
     cl_ld(a, ev);
     sh_st(x + e * W, xv + ev);
   }
-  cl_end(kind);
+  cl_end<KIND>();
 }
 
-template <typename R>
-__device__ __noinline__ void cl_zero(unsigned lv, int kind) {
-  cl_begin(kind);
-  const unsigned here = CL_F(lv, here), x = CL_F(lv, x), step = cl_step(kind);
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_zero(unsigned lv) {
+  cl_begin<KIND>();
+  const unsigned here = CL_F(lv, here), x = CL_F(lv, x), step = kClStep<KIND>;
   for (unsigned e = threadIdx.x; e < here; e += step) sh_st(x + e * (unsigned)sizeof(R), R(0));
-  cl_end(kind);
+  cl_end<KIND>();
 }
 
 // exact coarsest solve, one row of the inverse a thread (b and x in storage order)
@@ -377,46 +413,215 @@ __device__ __forceinline__ void coarse_solve(const R* cinv, const R* b, R* x, in
 
 // the same on the slots of the coarsest level; row i of the inverse starts at i (n + 1), so
 // that the rows of a warp fall into different banks
-template <typename R>
-__device__ __noinline__ void cl_coarse(unsigned lv, unsigned cinv, int kind) {
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_coarse(unsigned lv, unsigned cinv) {
   constexpr unsigned W = sizeof(R);
   const unsigned n = CL_F(lv, cells), b = CL_F(lv, b), x = CL_F(lv, x), res = CL_F(lv, res), ord = CL_F(lv, ord);
-  const unsigned step = cl_step(kind);
-  cl_begin(kind);
+  const unsigned step = kClStep<KIND>;
+  cl_begin<KIND>();
   // b to position order (res is free on the coarsest level)
   for (unsigned e = threadIdx.x; e < n; e += step) {
     R v;
     sh_ld(b + e * W, v);
     sh_st(res + sh_ld16(ord + e * 2u) * W, v);
   }
-  cl_begin(kind);
+  cl_begin<KIND>();
   for (unsigned e = threadIdx.x; e < n; e += step) {
     const unsigned row = cinv + sh_ld16(ord + e * 2u) * (n + 1) * W;
     R v = R(0);
-#pragma unroll 4
-    for (unsigned j = 0; j < n; j++) {
-      R bj, m;
-      sh_ld(res + j * W, bj);
+    unsigned j = 0;
+    for (; j + 8 <= n; j += 8) {  // eight products' loads in flight: the chain is the fma's 64 cycles each
+      R m[8], bj[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        sh_ld(row + (j + q) * W, m[q]);
+        sh_ld(res + (j + q) * W, bj[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; q++) v = fma_r(m[q], bj[q], v);
+    }
+    for (; j < n; j++) {
+      R m, bj;
       sh_ld(row + j * W, m);
+      sh_ld(res + j * W, bj);
       v = fma_r(m, bj, v);
     }
     sh_st(x + e * W, v);
   }
-  cl_end(kind);
+  cl_end<KIND>();
+}
+
+// most cells of one colour a thread may have in a descent or ascent: two with two neighbours
+// each (the first coarse levels of a column), else one
+__host__ __device__ constexpr int cl_per_thread(int ne) { return ne == 2 ? 2 : 1; }
+
+// A level's whole descent or ascent where every thread has at most cl_per_thread cells of a colour
+// (all levels but a few): coefficients, addresses and right-hand sides stay in registers
+// from one phase to the next, and a phase is a barrier, one round of loads, the fma chain
+// and a store.  The separate phases fetch them again each time: 640-830 cycles a half sweep
+// of one warp, of which 200-450 are FP64.
+// Lanes without a cell repeat slot 0 and store nothing; warps without one do nothing.
+template <typename R, int NE>
+struct ClCell {
+  unsigned e, nb[NE];
+  R k[NE], di;
+  bool ok, warp;  // this thread, this warp has a cell
+  __device__ __forceinline__ void fetch(unsigned from, unsigned last, unsigned cap, unsigned dinv, unsigned cf, unsigned na) {
+    constexpr unsigned W = sizeof(R);
+    const unsigned slot = from + threadIdx.x;
+    ok = slot < last;
+    warp = from + (threadIdx.x & ~31u) < last;
+    e = ok ? slot : 0u;
+    sh_ld(dinv + e * W, di);
+#pragma unroll
+    for (int d = 0; d < NE; d++) {
+      nb[d] = sh_ldw(na + (d * cap + e) * 4u);
+      sh_ld(cf + (d * cap + e) * W, k[d]);
+    }
+  }
+  __device__ __forceinline__ R sum(R v) const {
+    R xn[NE];
+#pragma unroll
+    for (int d = 0; d < NE; d++) cl_ld(nb[d], xn[d]);
+#pragma unroll
+    for (int d = 0; d < NE; d++) v = fma_r(k[d], xn[d], v);
+    return v;
+  }
+};
+
+template <typename R, int KIND, int NE>
+__device__ __forceinline__ void cl_down_one(unsigned lv, int nu1, int folded) {
+  constexpr unsigned W = sizeof(R);
+  constexpr int M = cl_per_thread(NE);
+  const unsigned cap = CL_F(lv, cap), red = CL_F(lv, red), here = CL_F(lv, here);
+  const unsigned x = CL_F(lv, x), b = CL_F(lv, b), dinv = CL_F(lv, dinv), cf = CL_F(lv, coef), nb = CL_F(lv, nb);
+  const unsigned diag = CL_F(lv, diag), rs = CL_F(lv, res), ord = CL_F(lv, ord);
+  ClCell<R, NE> c0[M], c1[M];
+  R dg[M], b0[M], b1[M];
+  unsigned res[M];
+#pragma unroll
+  for (int m = 0; m < M; m++) {
+    c0[m].fetch(m * kClStep<KIND>, red, cap, dinv, cf, nb);
+    c1[m].fetch(red + m * kClStep<KIND>, here, cap, dinv, cf, nb);
+    sh_ld(diag + c0[m].e * W, dg[m]);
+    res[m] = rs + sh_ld16(ord + c0[m].e * 2u) * W;
+  }
+  cl_begin<KIND>();
+#pragma unroll
+  for (int m = 0; m < M; m++) {
+    sh_ld(b + c0[m].e * W, b0[m]);
+    sh_ld(b + c1[m].e * W, b1[m]);
+  }
+  if (!folded) {
+#pragma unroll
+    for (int m = 0; m < M; m++)
+      if (c0[m].warp) sh_st_if(x + c0[m].e * W, b0[m] * c0[m].di, c0[m].ok);
+    cl_end<KIND>();
+    cl_begin<KIND>();
+  }
+  for (int it = 0;; it++) {
+#pragma unroll
+    for (int m = 0; m < M; m++)
+      if (c1[m].warp) sh_st_if(x + c1[m].e * W, c1[m].sum(b1[m]) * c1[m].di, c1[m].ok);
+    cl_end<KIND>();
+    cl_begin<KIND>();
+    if (it + 1 >= nu1) break;
+#pragma unroll
+    for (int m = 0; m < M; m++)
+      if (c0[m].warp) sh_st_if(x + c0[m].e * W, c0[m].sum(b0[m]) * c0[m].di, c0[m].ok);
+    cl_end<KIND>();
+    cl_begin<KIND>();
+  }
+#pragma unroll
+  for (int m = 0; m < M; m++)
+    if (c0[m].warp) {
+      R xo;
+      sh_ld(x + c0[m].e * W, xo);
+      const R v = c0[m].sum(R(0));
+      sh_st_if(res[m], b0[m] - (mul_r(dg[m], xo) - v), c0[m].ok);
+    }
+  cl_end<KIND>();
+}
+
+template <typename R, int KIND, int NE>
+__device__ __forceinline__ void cl_up_one(unsigned lv, int nu2) {
+  constexpr unsigned W = sizeof(R);
+  constexpr int M = cl_per_thread(NE);
+  const unsigned cap = CL_F(lv, cap), red = CL_F(lv, red), here = CL_F(lv, here);
+  const unsigned x = CL_F(lv, x), b = CL_F(lv, b), dinv = CL_F(lv, dinv), cf = CL_F(lv, coef), nb = CL_F(lv, nb);
+  const unsigned pa = CL_F(lv, par);
+  ClCell<R, NE> c0[M], c1[M];
+  R b0[M], b1[M], xo[M];
+  unsigned par[M];
+#pragma unroll
+  for (int m = 0; m < M; m++) {
+    c0[m].fetch(m * kClStep<KIND>, red, cap, dinv, cf, nb);
+    c1[m].fetch(red + m * kClStep<KIND>, here, cap, dinv, cf, nb);
+    sh_ld(b + c0[m].e * W, b0[m]);
+    par[m] = sh_ldw(pa + c0[m].e * 4u);
+    sh_ld(b + c1[m].e * W, b1[m]);
+  }
+  cl_begin<KIND>();
+#pragma unroll
+  for (int m = 0; m < M; m++)
+    if (c0[m].warp) {
+      R ev;
+      cl_ld(par[m], ev);
+      sh_ld(x + c0[m].e * W, xo[m]);
+      sh_st_if(x + c0[m].e * W, xo[m] + ev, c0[m].ok);
+    }
+  cl_end<KIND>();
+  for (int it = 0; it < nu2; it++) {
+    cl_begin<KIND>();
+#pragma unroll
+    for (int m = 0; m < M; m++)
+      if (c1[m].warp) sh_st_if(x + c1[m].e * W, c1[m].sum(b1[m]) * c1[m].di, c1[m].ok);
+    cl_end<KIND>();
+    cl_begin<KIND>();
+#pragma unroll
+    for (int m = 0; m < M; m++)
+      if (c0[m].warp) sh_st_if(x + c0[m].e * W, c0[m].sum(b0[m]) * c0[m].di, c0[m].ok);
+    cl_end<KIND>();
+  }
+}
+
+template <int KIND>
+__device__ __forceinline__ bool cl_fits(unsigned lv) {
+  return CL_F(lv, most) <= kClStep<KIND> * (unsigned)cl_per_thread((int)CL_F(lv, ne));
 }
 
 // pre-smoothing and residual of a level (its b is complete; folded: its zero-guess
 // colour-0 update came with b)
-template <typename R>
-__device__ __forceinline__ void cl_down(unsigned lv, int nu1, int folded, int kind) {
-  if (nu1 == 0) cl_zero<R>(lv, kind);
-  for (int h = folded ? 1 : 0; h < 2 * nu1; h++) cl_half<R>(lv, h & 1, h == 0, kind);
-  cl_resid<R>(lv, nu1 > 0 ? 1 : 0, kind);
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_down(unsigned lv, int nu1, int folded) {
+  if (nu1 > 0 && cl_fits<KIND>(lv)) {
+    const unsigned ne = CL_F(lv, ne);
+    if (ne == 6)
+      cl_down_one<R, KIND, 6>(lv, nu1, folded);
+    else if (ne == 4)
+      cl_down_one<R, KIND, 4>(lv, nu1, folded);
+    else
+      cl_down_one<R, KIND, 2>(lv, nu1, folded);
+    return;
+  }
+  if (nu1 == 0) cl_zero<R, KIND>(lv);
+  for (int h = folded ? 1 : 0; h < 2 * nu1; h++) cl_half<R, KIND>(lv, h & 1, h == 0);
+  cl_resid<R, KIND>(lv, nu1 > 0 ? 1 : 0);
 }
-template <typename R>
-__device__ __forceinline__ void cl_up(unsigned lv, int nu2, int kind) {
-  cl_prolong<R>(lv, nu2 > 0 ? 1 : 0, kind);
-  for (int h = 0; h < 2 * nu2; h++) cl_half<R>(lv, 1 - (h & 1), 0, kind);
+template <typename R, int KIND>
+__device__ __forceinline__ void cl_up(unsigned lv, int nu2) {
+  if (nu2 > 0 && cl_fits<KIND>(lv)) {
+    const unsigned ne = CL_F(lv, ne);
+    if (ne == 6)
+      cl_up_one<R, KIND, 6>(lv, nu2);
+    else if (ne == 4)
+      cl_up_one<R, KIND, 4>(lv, nu2);
+    else
+      cl_up_one<R, KIND, 2>(lv, nu2);
+    return;
+  }
+  cl_prolong<R, KIND>(lv, nu2 > 0 ? 1 : 0);
+  for (int h = 0; h < 2 * nu2; h++) cl_half<R, KIND>(lv, 1 - (h & 1), 0);
 }
 
 // the levels in CTA 0 from level l0 on, called by all its threads; ends with a block barrier
@@ -426,26 +631,29 @@ __device__ __forceinline__ void cl_solo(const Cl<R>& c, int l0, int nlev, int nu
   int lw = l0;  // first level of the single warp
   while (lw < lc && CL_F(c.level(lw), cells) > kClWarp) lw++;
   for (int l = l0; l < lw; l++) {
-    cl_down<R>(c.level(l), nu1, l == l0 ? folded : mask, kByBlock);
-    cl_gather<R>(c.level(l + 1), mask, kByBlock);
+    cl_down<R, kByBlock>(c.level(l), nu1, l == l0 ? folded : mask);
+    cl_gather<R, kByBlock>(c.level(l + 1), mask);
   }
   __syncthreads();
   if (threadIdx.x < 32) {
     for (int l = lw; l < lc; l++) {
-      cl_down<R>(c.level(l), nu1, l == l0 ? folded : mask, kByWarp);
-      cl_gather<R>(c.level(l + 1), mask, kByWarp);
+      cl_down<R, kByWarp>(c.level(l), nu1, l == l0 ? folded : mask);
+      cl_gather<R, kByWarp>(c.level(l + 1), mask);
     }
-    for (int h = 0; h < 2 * cs; h++) cl_half<R>(c.level(lc), h & 1, h == 0, kByWarp);
-    for (int h = 0; h < 2 * cs; h++) cl_half<R>(c.level(lc), 1 - (h & 1), 0, kByWarp);
+    for (int h = 0; h < 2 * cs; h++) cl_half<R, kByWarp>(c.level(lc), h & 1, h == 0);
+    for (int h = 0; h < 2 * cs; h++) cl_half<R, kByWarp>(c.level(lc), 1 - (h & 1), 0);
   }
   if (cs == 0) {
     const bool wide = CL_F(c.level(lc), cells) > 32;
-    if (wide || threadIdx.x < 32) cl_coarse<R>(c.level(lc), c.cinv, wide ? kByBlock : kByWarp);
+    if (wide)
+      cl_coarse<R, kByBlock>(c.level(lc), c.cinv);
+    else if (threadIdx.x < 32)
+      cl_coarse<R, kByWarp>(c.level(lc), c.cinv);
     if (wide) __syncthreads();
   }
   if (threadIdx.x < 32)
-    for (int l = lc - 1; l >= lw; l--) cl_up<R>(c.level(l), nu2, kByWarp);
-  for (int l = lw - 1; l >= l0; l--) cl_up<R>(c.level(l), nu2, kByBlock);
+    for (int l = lc - 1; l >= lw; l--) cl_up<R, kByWarp>(c.level(l), nu2);
+  for (int l = lw - 1; l >= l0; l--) cl_up<R, kByBlock>(c.level(l), nu2);
   __syncthreads();
 }
 
@@ -454,21 +662,21 @@ __device__ __forceinline__ void cl_solo(const Cl<R>& c, int l0, int nlev, int nu
 // arrived at the cluster barrier, and waits for the last half sweep's arrival; otherwise
 // everything happens in CTA 0 between block barriers.
 template <typename R>
-__device__ __noinline__ void cl_vcycle(Cl<R> c, int first, int nlev, int nu1, int nu2, int cs) {
+__device__ __forceinline__ void cl_vcycle(Cl<R> c, int first, int nlev, int nu1, int nu2, int cs) {
   const int mask = nu1 > 0 ? 1 : 0;
   int ls = first;  // first level in CTA 0
   while (!CL_F(c.level(ls), solo)) ls++;
   for (int l = first; l < ls; l++) {
-    cl_down<R>(c.level(l), nu1, l == first ? 0 : mask, kByCluster);
-    if (l + 1 < ls) cl_gather<R>(c.level(l + 1), mask, kByCluster);
+    cl_down<R, kByCluster>(c.level(l), nu1, l == first ? 0 : mask);
+    if (l + 1 < ls) cl_gather<R, kByCluster>(c.level(l + 1), mask);
   }
   if (ls > first) cl_wait();
   if (c.rank == 0) {
-    if (ls > first) cl_gather<R>(c.level(ls), mask, kByBlock);
+    if (ls > first) cl_gather<R, kByBlock>(c.level(ls), mask);
     cl_solo<R>(c, ls, nlev, nu1, nu2, cs, ls > first ? mask : 0);
   }
   if (ls > first) cl_arrive();
-  for (int l = ls - 1; l >= first; l--) cl_up<R>(c.level(l), nu2, kByCluster);
+  for (int l = ls - 1; l >= first; l--) cl_up<R, kByCluster>(c.level(l), nu2);
 }
 
 // Level table, coefficients, slots and neighbour addresses of levels first .. nlev - 1.
@@ -524,7 +732,11 @@ __device__ void cl_setup(Cl<R>& c, ClLevel* lv, Level<R>* gl, unsigned sm, const
   }
   cl_arrive();
   cl_wait();
-  if ((int)tid >= first && (int)tid < nlev) lv[tid].red = s_count[0][tid];
+  if ((int)tid >= first && (int)tid < nlev) {
+    const int r = s_count[0][tid], k = lv[tid].here - r;
+    lv[tid].red = r;
+    lv[tid].most = r > k ? r : k;
+  }
   for (int f = (int)tid; f < total; f += kClThreads) {
     int l = first;
     while (f >= s_off[l + 1]) l++;
@@ -647,7 +859,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
 template <typename R, int ROWS>
 __global__ void __launch_bounds__(kClThreads, 1)
     k_cg_cluster(const StepDom* __restrict__ D, const CgDom* __restrict__ CG, const int* __restrict__ idx, int ctas,
-                 int nu1, int nu2, int cs, double tol, int max_it) {
+                 int nu1, int nu2, int cs, double tol, int max_it, int early) {
   constexpr bool kFlex = std::is_same<R, float>::value;
   constexpr unsigned W = sizeof(R);
   extern __shared__ __align__(16) unsigned char cl_sm[];
@@ -662,8 +874,11 @@ __global__ void __launch_bounds__(kClThreads, 1)
   Cl<R> c{sh_addr(lv), blockIdx.x % ctas, 0u};
   unsigned end;
   const int nlev = G.nlev;
-  // the wait comes first: the operator's build may be the preceding kernel
-  MDBS_DEPENDENT_ENTRY();
+  // A step's first solve waits here: the operator's build may be among the kernels it follows
+  // (the branch it runs on joins ahead of this kernel, and a captured join can be a
+  // programmatic dependency like any other).  In the later ones, which follow the first, the
+  // setup overlaps the preceding kernel; all it reads is the operator.
+  if (!early) MDBS_PDL_WAIT();
   cl_setup<R>(c, lv, gl, sh_addr(cl_sm), G, 0, nlev, ctas, ROWS, nu1 > 0 ? 1 : 0, &end);
   const unsigned db = end;  // the vector A is applied to, exchanged through the cluster
 
@@ -693,8 +908,6 @@ __global__ void __launch_bounds__(kClThreads, 1)
     nat[w] = (unsigned)q[0] + (unsigned)S.P.n[0] * ((unsigned)q[1] + (unsigned)S.P.n[1] * (unsigned)q[2]);
     slot[w] = sh_ld16(L0.res + e * W);  // still the slots of cl_setup
     dg[w] = S.F.diag[pos];
-    bc[w] = S.F.b[pos];
-    p[w] = S.F.p[nat[w]];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
       const bool has_lo = q[d] > 0, has_hi = q[d] + 1 < S.P.n[d];
@@ -705,6 +918,14 @@ __global__ void __launch_bounds__(kClThreads, 1)
       na[w][2 * d + 1] = cl_map(db + cl_local(L0, ph) * 8u, cl_owner(L0, ph));
     }
   }
+  if (early) MDBS_PDL_WAIT();
+  MDBS_PDL_TRIGGER();
+#pragma unroll
+  for (int w = 0; w < ROWS; w++)
+    if (in[w]) {
+      bc[w] = S.F.b[cl_position(L0, c.rank, w * kClThreads + t)];
+      p[w] = S.F.p[nat[w]];
+    }
   auto sync_all = [&] {
     if (ctas > 1) {
       cl_arrive();

@@ -2572,7 +2572,7 @@ cudaError_t pressure_solve(const BatchPlan& B, double tol, int max_it, int nu1, 
     prof_begin(K_CG_CLUSTER, s);
     auto launch = [&](auto kernel) {
       return launch_cluster(kernel, B.n_small, B.small_ctas, B.small_smem, s, B.sd, B.cg, B.small_idx, B.small_ctas, nu1,
-                            nu2, cs, tol, max_it);
+                            nu2, cs, tol, max_it, corr > 0 ? 1 : 0);
     };
     const int rows = B.small_rows;
     const cudaError_t le = flexible ? (rows == 1   ? launch(k_cg_cluster<float, 1>)
