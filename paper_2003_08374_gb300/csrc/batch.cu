@@ -62,18 +62,17 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
     return (int)acc;
   };
   int totals[6 + 7 * kMaxLevels];
-  // one row of kBlock elements per item, except the reduction spaces (kRepBig rows:
+  // one row of kBlock elements per item, except the reduction spaces (StepDom::rep rows:
   // fewer block reductions and partials)
   int reps[6 + 7 * kMaxLevels];
   for (int q = 0; q < nspace; q++) reps[q] = 1;
-  reps[3] = reps[4] = kRepBig;
   reps[5 + kMaxLevels] = smooth_rows;  // finest-level red/black half sweeps
   auto blocks_of = [&](long long n, int space) { return items_of(n, reps[space]); };
   totals[0] = fill(0, [&](int d) { return blocks_of(sd[d].P.cells, 0); });
   totals[1] = fill(1, [&](int d) { return blocks_of(faces_total(sd[d].P), 1); });
   totals[2] = fill(2, [&](int) { return 1LL; });
-  totals[3] = fill(3, [&](int d) { return blocks_of(sd[d].P.cells, 3); });
-  totals[4] = fill(4, [&](int d) { return blocks_of(faces_total(sd[d].P), 4); });
+  totals[3] = fill(3, [&](int d) { return red_items(sd[d].P.cells, sd[d].rep); });
+  totals[4] = fill(4, [&](int d) { return red_items(faces_total(sd[d].P), sd[d].rep); });
   totals[scg] = fill(scg, [&](int d) { return cg[d].small ? 0LL : cg_items(sd[d].P.cells); });
   B.max_first = 0;
   B.max_levels = 0;
@@ -96,7 +95,9 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
       return (long long)L.n[0] * L.n[1] * L.n[2];
     };
     const int s0 = 5 + l, s1 = 5 + kMaxLevels + l, s2 = 5 + 2 * kMaxLevels + l, s3 = 5 + 3 * kMaxLevels + l;
-    totals[s0] = fill(s0, [&](int d) { return l < cg[d].nlev ? blocks_of(cells_at(d, l), s0) : 0LL; });
+    totals[s0] = fill(s0, [&](int d) {
+      return l < cg[d].nlev && cells_at(d, l) > kBuildCells ? blocks_of(cells_at(d, l), s0) : 0LL;
+    });
     totals[s1] = fill(s1, [&](int d) -> long long {
       if (l >= cg[d].first) return 0;
       const Level<double>& L = cg[d].ld[l];

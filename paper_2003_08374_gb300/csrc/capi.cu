@@ -297,7 +297,7 @@ size_t carve(mdbs_sim* s, const Layout& L, char* base) {
     F.gphi[d] = (double*)take(3 * nf * 8);
   }
   const long long faces = L.nf[0] + L.nf[1] + (L.dim == 3 ? L.nf[2] : 0);
-  const long long pcap = (std::max(L.cells, faces) + kBlock * kRepBig - 1) / (kBlock * kRepBig);
+  const long long pcap = red_items(std::max(L.cells, faces), red_rep(L.cells, faces));
   double* partials = (double*)take(4 * pcap * 8);
   double* scal = (double*)take(kNumSlots * 8);
   if (s) {
@@ -372,6 +372,7 @@ StepDom step_view(const mdbs_sim* s) {
   d.scal = s->scal;
   d.partials = s->partials;
   d.pcap = s->pcap;
+  d.rep = red_rep(s->P.cells, s->P.nf[0] + s->P.nf[1] + (s->P.dim == 3 ? s->P.nf[2] : 0));
   return d;
 }
 

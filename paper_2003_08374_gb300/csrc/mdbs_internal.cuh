@@ -147,6 +147,7 @@ struct StepDom {
   double* scal;      // step scalars (kSlot*)
   double* partials;  // reduction partials: 4 channels of pcap values
   long long pcap;    // partials per channel (>= work items of the largest space)
+  int rep;           // rows of kBlock elements per item of the reduction spaces (red_rep)
 };
 
 // per-domain view of the pressure solver
@@ -183,7 +184,18 @@ struct CgVec {
   double* scal;
 };
 
+// Rows of kBlock elements per item of a domain's other reductions (saturation flux, CFL number,
+// statistics): one while that is at most two waves of resident blocks (the saturation flux of
+// 64^2 cells took 37 us in 5 blocks), else kRepBig.  A property of the domain, so that its
+// sums are the same alone and in any batch.
+__host__ __device__ inline int red_rep(long long cells, long long faces) {
+  const long long most = faces > cells ? faces : cells;
+  return most <= 2432LL * kBlock ? 1 : kRepBig;
+}
+inline long long red_items(long long n, int rep) { return (n + (long long)kBlock * rep - 1) / ((long long)kBlock * rep); }
+
 // partial sums of a domain's CG reductions: kRepBig rows of kBlock cells each
+constexpr int kBuildCells = 512;  // levels up to this size are built by one block per domain (k_build_small)
 inline long long cg_items(long long cells) { return (cells + kBlock * kRepBig - 1) / (kBlock * kRepBig); }
 
 // ---------------------------------------------------------------- helpers
@@ -322,7 +334,7 @@ struct BatchPlan {
   size_t small_smem;          // its dynamic shared memory
   int cl_tail_ctas;           // > 0: the tails run in clusters of this many CTAs
   size_t cl_tail_smem;
-  Work lcells[kMaxLevels];    // level-l cells of domains that have level l
+  Work lcells[kMaxLevels];    // level-l cells of domains that have level l, of more than kBuildCells cells
   Work lhalf[kMaxLevels];     // level-l red/black half cells of domains whose level l precedes the tail
   Work lfine[kMaxLevels];     // level-l cells of the same domains (prolongation)
   Work lcoarse[kMaxLevels];   // level-(l+1) cells of the same domains (restriction phase of the cooperative kernel)
@@ -393,7 +405,6 @@ void pressure_view(const PressureSolver* ps, const Fld& F, int tail_cells, CgDom
 void pressure_storage(const PressureSolver* ps, void** ptr, size_t* bytes);
 constexpr int kTailCellsMax = 262144;
 int pressure_precision(const PressureSolver* ps);
-constexpr int kAsmMatrix = 1, kAsmRhs = 2;
 void launch_pressure_matrix(const BatchPlan& B, int coarse_sweeps, cudaStream_t s);
 void launch_pressure_rhs(const BatchPlan& B, cudaStream_t s);
 // Enqueues the solve of A p = b for every domain of the batch by GMG-preconditioned

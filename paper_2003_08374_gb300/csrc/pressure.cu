@@ -139,131 +139,147 @@ constexpr int kBB = 0, kRR = 1, kRZ = 2, kDQ = 3, kZQ = 4, kAlpha = 5, kCond = 6
     const int dm = work_domain((W), b_);                                  \
     const int lb = b_ - (W).blk[dm];
 
+// a product that is rounded by itself
+__device__ __forceinline__ double mul_r(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b); }
+
 // ------------------------------------------------------------------ assembly
 // T_f = A^2 / a_P,f between cells, 2 A^2 / a_P,f on outlet faces (Dirichlet
 // through the ghost p_ghost = -p), b = -sum_f s_f A ubar_f with ubar = HbyA on
 // unknown faces and the fixed velocity on wall / inlet faces.
-// what: kAsmMatrix (coefficients T, Dd) and / or kAsmRhs (right-hand side b)
-__device__ __forceinline__ void b_assemble(const Prm& P, const Fld& F, long long c, int what) {
-  const bool matrix = what & kAsmMatrix;
+__device__ __forceinline__ void b_rhs(const Prm& P, const Fld& F, long long c) {
   int q[3];
   decode_pos(P, c, q[0], q[1], q[2]);  // c: storage position of the cell
-  const double A = P.A, A2 = P.A * P.A;
-  double div = 0.0, Dd = 0.0;
+  const double A = P.A;
+  double div = 0.0;
+#pragma unroll
   for (int d = 0; d < 3; d++) {
-    if (d >= P.dim) {
-      if (matrix) F.T[d][c] = 0.0;
-      continue;
-    }
+    if (d >= P.dim) continue;
     const int di = (d == 0), dj = (d == 1), dk = (d == 2);
     const long long flo = face_index(P.n, d, q[0], q[1], q[2]);
     const long long fhi = face_index(P.n, d, q[0] + di, q[1] + dj, q[2] + dk);
-    if (matrix) F.T[d][c] = (q[d] + 1 < P.n[d]) ? A2 * F.aP[d][fhi] : 0.0;  // aP holds 1 / a_P
-    const bool lo_bnd = q[d] == 0, hi_bnd = q[d] + 1 == P.n[d];
-    if (lo_bnd && P.bc[2 * d] == kOutlet) Dd += 2.0 * A2 * F.aP[d][flo];
-    if (hi_bnd && P.bc[2 * d + 1] == kOutlet) Dd += 2.0 * A2 * F.aP[d][fhi];
-    const bool lo_fixed = lo_bnd && P.bc[2 * d] != kOutlet;
-    const bool hi_fixed = hi_bnd && P.bc[2 * d + 1] != kOutlet;
+    const bool lo_fixed = q[d] == 0 && P.bc[2 * d] != kOutlet;
+    const bool hi_fixed = q[d] + 1 == P.n[d] && P.bc[2 * d + 1] != kOutlet;
     const double ulo = lo_fixed ? F.u[d][flo] : F.hbya[d][flo];
     const double uhi = hi_fixed ? F.u[d][fhi] : F.hbya[d][fhi];
     div += A * uhi - A * ulo;
   }
-  if (matrix) F.Dd[c] = Dd;
-  if (what & kAsmRhs) F.b[c] = -div;
+  F.b[c] = -div;
 }
 
-__global__ void k_assemble(const StepDom* __restrict__ D, Work w, int what) {
+__global__ void k_rhs(const StepDom* __restrict__ D, Work w) {
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK(w)
     const StepDom& S = D[dm];
     for (int r = 0; r < w.rep; r++) {
       const long long c = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
-      if (c < S.P.cells) b_assemble(S.P, S.F, c, what);
+      if (c < S.P.cells) b_rhs(S.P, S.F, c);
     }
   }
 }
 
-template <typename R>
-__device__ __forceinline__ R coef_lo(const Level<R>& L, int d, const int q[3], long long c) {
-  if (q[d] == 0) return R(0);
-  return tcoef(L, d, lo_pos(L.n, q, (unsigned)c, d));
-}
-
-template <typename R>
-__device__ __forceinline__ void b_diag(const Level<R>& L, long long c) {
-  int q[3];
-  decode_pos(L, c, q[0], q[1], q[2]);
-  R dg = R(0);
-  for (int d = 0; d < 3; d++) {
-    dg += tcoef(L, d, (unsigned)c);
-    if (q[d] > 0) dg += coef_lo(L, d, q, c);
-  }
-  const R dgt = dg + L.Dd[c];
-  L.diag[c] = dgt;
-  L.dinv[c] = R(1) / dgt;
-}
-
-template <typename R>
-__global__ void k_diag(const CgDom* __restrict__ C, Work w, int l) {
+// The finest operator in one pass: T, D, the diagonal and its reciprocal, and in mixed
+// precision their FP32 copies.  A cell forms the coefficients of its lower faces too (the
+// products its neighbours store), so the diagonal needs no second pass over T (three passes
+// before: 16.8 M cells, 0.37 + 0.28 + 0.21 ms).
+template <bool FLEX>
+__global__ void k_operator(const StepDom* __restrict__ D, const CgDom* __restrict__ C, Work w) {
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK(w)
-    const Level<R>& L = levels_of<R>(C[dm])[l];
+    const StepDom& S = D[dm];
+    const Prm& P = S.P;
+    const Fld& F = S.F;
     for (int r = 0; r < w.rep; r++) {
       const long long c = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
-      if (c < L.cells) b_diag(L, c);
-    }
-  }
-}
-
-// FP32 copy of the level-0 operator (mixed precision), with its reciprocal diagonal
-__global__ void k_level0_to_float(const CgDom* __restrict__ C, Work w) {
-  MDBS_DEPENDENT_ENTRY();
-  FOR_WORK(w)
-    const Level<double>& Ld = C[dm].ld[0];
-    const Level<float>& Lf = C[dm].lf[0];
-    for (int r = 0; r < w.rep; r++) {
-      const long long c = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
-      if (c < Ld.cells) {
-        for (int a = 0; a < 3; a++) Lf.T[a][c] = (float)Ld.T[a][c];
-        Lf.Dd[c] = (float)Ld.Dd[c];
-        const float dg = (float)Ld.diag[c];
-        Lf.diag[c] = dg;
-        Lf.dinv[c] = 1.0f / dg;
+      if (c >= P.cells) continue;
+      int q[3];
+      decode_pos(P, c, q[0], q[1], q[2]);  // c: storage position of the cell
+      const double A2 = P.A * P.A;
+      double Dd = 0.0, dg = 0.0, t[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int d = 0; d < 3; d++) {
+        if (d < P.dim) {
+          const long long flo = face_index(P.n, d, q[0], q[1], q[2]);
+          const long long fhi = face_index(P.n, d, q[0] + (d == 0), q[1] + (d == 1), q[2] + (d == 2));
+          const bool lo_bnd = q[d] == 0, hi_bnd = q[d] + 1 == P.n[d];
+          if (!hi_bnd) t[d] = mul_r(A2, F.aP[d][fhi]);  // aP holds 1 / a_P
+          if (lo_bnd && P.bc[2 * d] == kOutlet) Dd += 2.0 * A2 * F.aP[d][flo];
+          if (hi_bnd && P.bc[2 * d + 1] == kOutlet) Dd += 2.0 * A2 * F.aP[d][fhi];
+          dg += t[d];
+          if (!lo_bnd) dg += mul_r(A2, F.aP[d][flo]);
+        }
+        F.T[d][c] = t[d];
+      }
+      const double dgt = dg + Dd;
+      F.Dd[c] = Dd;
+      F.diag[c] = dgt;
+      F.dinv[c] = 1.0 / dgt;
+      if (FLEX) {
+        const Level<float>& Lf = C[dm].lf[0];
+        for (int a = 0; a < 3; a++) Lf.T[a][c] = (float)t[a];
+        Lf.Dd[c] = (float)Dd;
+        const float df = (float)dgt;
+        Lf.diag[c] = df;
+        Lf.dinv[c] = 1.0f / df;
       }
     }
   }
 }
 
-// coarse transmissibilities: the sum of the fine links crossing the coarse face
-// (the Galerkin operator of piecewise-constant transfer), halved when the face's
-// normal axis is coarsened, where the 2h link spans twice the fine distance
+// Coarse transmissibility of the upper face of coarse cell Q along d: the sum of the fine
+// links crossing it (the Galerkin operator of piecewise-constant transfer), halved when the
+// face's normal axis is coarsened, where the 2h link spans twice the fine distance; as it is
+// stored (rounded to BF16 where the level stores that)
+template <typename R>
+__device__ __forceinline__ R coarse_link(const Level<R>& Fi, const Level<R>& Co, const int Q[3], int d) {
+  int rl[3], rh[3];
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const int last = Co.cz[a] ? 2 * Q[a] + 1 : Q[a];  // last fine cell of coarse cell Q
+    rl[a] = a == d ? last : (Co.cz[a] ? 2 * Q[a] : Q[a]);
+    rh[a] = a == d || last < Fi.n[a] ? last : last - 1;
+  }
+  R sum = R(0);
+  for (int z = rl[2]; z <= rh[2]; z++)
+    for (int y = rl[1]; y <= rh[1]; y++)
+      for (int x = rl[0]; x <= rh[0]; x++) sum += tcoef(Fi, d, (unsigned)lpos(Fi.n, x, y, z));
+  const R v = Co.cz[d] ? R(0.5) * sum : sum;
+  if constexpr (std::is_same<R, float>::value)
+    if (Co.Tb[d]) return __bfloat162float(__float2bfloat16_rn(v));
+  return v;
+}
+
+// Cell ci of a coarse level: its links, the outlet term, the diagonal and its reciprocal.  The
+// links of its lower faces, which its neighbours store, are formed again for the diagonal, so
+// that a level is one pass (and one launch).
 template <typename R>
 __device__ __forceinline__ void b_coarsen(const Level<R>& Fi, const Level<R>& Co, long long ci) {
   int Q[3];
   decode_pos(Co, ci, Q[0], Q[1], Q[2]);
+  R dg = R(0);
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const R up = Q[d] + 1 < Co.n[d] ? coarse_link(Fi, Co, Q, d) : R(0);
+    tstore(Co, d, (unsigned)ci, up);
+    dg += up;
+    if (Q[d] > 0) {
+      const int L[3] = {Q[0] - (d == 0), Q[1] - (d == 1), Q[2] - (d == 2)};
+      dg += coarse_link(Fi, Co, L, d);
+    }
+  }
   int lo[3], hi[3];
   for (int a = 0; a < 3; a++) {
     lo[a] = Co.cz[a] ? 2 * Q[a] : Q[a];
     hi[a] = Co.cz[a] ? (2 * Q[a] + 1 < Fi.n[a] ? 2 * Q[a] + 1 : 2 * Q[a]) : Q[a];
-  }
-  for (int d = 0; d < 3; d++) {
-    if (Q[d] + 1 >= Co.n[d]) {
-      tstore(Co, d, (unsigned)ci, R(0));
-      continue;
-    }
-    int rl[3] = {lo[0], lo[1], lo[2]}, rh[3] = {hi[0], hi[1], hi[2]};
-    rl[d] = rh[d] = Co.cz[d] ? 2 * Q[d] + 1 : Q[d];  // last fine cell of coarse cell Q
-    R sum = R(0);
-    for (int z = rl[2]; z <= rh[2]; z++)
-      for (int y = rl[1]; y <= rh[1]; y++)
-        for (int x = rl[0]; x <= rh[0]; x++) sum += tcoef(Fi, d, (unsigned)lpos(Fi.n, x, y, z));
-    tstore(Co, d, (unsigned)ci, Co.cz[d] ? R(0.5) * sum : sum);
   }
   R dd = R(0);
   for (int z = lo[2]; z <= hi[2]; z++)
     for (int y = lo[1]; y <= hi[1]; y++)
       for (int x = lo[0]; x <= hi[0]; x++) dd += R(0.5) * Fi.Dd[lpos(Fi.n, x, y, z)];
   Co.Dd[ci] = dd;
+  const R dgt = dg + dd;
+  Co.diag[ci] = dgt;
+  Co.dinv[ci] = R(1) / dgt;
 }
 
 template <typename R>
@@ -294,9 +310,6 @@ __device__ __forceinline__ R ldc(const R* p) {
 // fma chain, so no value depends on the compiler's contraction choices)
 __device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
-// a product that is rounded by itself
-__device__ __forceinline__ double mul_r(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b); }
 
 // b - A x at cell q (position c): the neighbour products in the order x-, x+, y-, y+, z-,
 // z+ from zero, then b - (diag x - sum) with the product rounded
@@ -1145,14 +1158,20 @@ __device__ __forceinline__ double* coarse_inverse_of<double>(const CgDom& G) { r
 template <>
 __device__ __forceinline__ float* coarse_inverse_of<float>(const CgDom& G) { return G.cinv_f; }
 
-// one block per domain
+constexpr int kBuildThreads = 1024;
+
+// Gauss-Jordan inverse of level C's operator in one block, without pivoting (the matrix is
+// symmetric positive definite).  Thread t keeps column t % 64 of rows t / 64, + 16, ...: its
+// column's scaled pivot entry is formed once a pivot for all its rows (with one entry after
+// another it was formed for each of them: 257 us for 64 cells, 74 for 36).  Per pivot every
+// thread reads what its entries need, a barrier, all write, a barrier; the thread that owns
+// the next diagonal entry forms that pivot's reciprocal from its new value before the first
+// barrier (double buffered: one FP64 division a pivot).
 template <typename R>
-__global__ void k_coarse_inverse(const CgDom* __restrict__ CG) {
-  MDBS_DEPENDENT_ENTRY();
-  const CgDom& G = CG[blockIdx.x];
-  const Level<R> C = levels_of<R>(G)[G.nlev - 1];
-  R* __restrict__ inv = coarse_inverse_of<R>(G);
+__device__ __forceinline__ void coarse_inverse(const Level<R>& C, R* __restrict__ inv) {
+  static_assert(kCoarseMax == 64 && kBuildThreads == 1024, "thread map");
   __shared__ R M[kCoarseMax * kCoarseMax];
+  __shared__ R piv[2];
   const int n = (int)C.cells;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) M[e] = R(0);
   __syncthreads();
@@ -1168,47 +1187,57 @@ __global__ void k_coarse_inverse(const CgDom* __restrict__ CG) {
       }
     }
   }
-  // Gauss-Jordan elimination without pivoting (the matrix is symmetric positive
-  // definite).  Each thread keeps the (row, column) of its entries (the launch has
-  // 1024 threads); per pivot every thread reads what its entries need, a barrier,
-  // all write, a barrier.  The thread that owns the next diagonal entry forms that
-  // pivot's reciprocal from its new value before the first barrier (double buffered:
-  // one FP64 division a pivot).
-  constexpr int kPer = (kCoarseMax * kCoarseMax + 1023) / 1024;
-  __shared__ R piv[2];
-  int ei[kPer], ej[kPer];
-  for (int t = 0; t < kPer; t++) {
-    const int e = threadIdx.x + t * blockDim.x;
-    ei[t] = e < n * n ? e / n : -1;
-    ej[t] = e < n * n ? e - ei[t] * n : -1;
-  }
-  if (threadIdx.x == 0) piv[0] = R(1) / M[0];
+  constexpr int kPer = 4;
+  const int j = threadIdx.x & 63, i0 = threadIdx.x >> 6;
+  if (threadIdx.x == 0) piv[0] = R(1) / C.diag[0];
   __syncthreads();
   for (int k = 0; k < n; k++) {
     const R pinv = piv[k & 1];
     R nv[kPer];
-    for (int t = 0; t < kPer; t++) {
-      const int i = ei[t], j = ej[t];
-      if (i < 0) continue;
-      if (i == k && j == k)
-        nv[t] = pinv;
-      else if (i == k)
-        nv[t] = M[k * n + j] * pinv;
-      else if (j == k)
-        nv[t] = -M[i * n + k] * pinv;
-      else
-        nv[t] = M[i * n + j] - M[i * n + k] * (M[k * n + j] * pinv);
-      if (i == k + 1 && j == k + 1) piv[(k + 1) & 1] = R(1) / nv[t];
+    if (j < n) {
+      const R tj = M[k * n + j] * pinv;
+#pragma unroll
+      for (int q = 0; q < kPer; q++) {
+        const int i = i0 + 16 * q;
+        if (i >= n) continue;
+        if (i == k)
+          nv[q] = j == k ? pinv : tj;
+        else if (j == k)
+          nv[q] = -M[i * n + k] * pinv;
+        else
+          nv[q] = M[i * n + j] - M[i * n + k] * tj;
+        if (i == k + 1 && j == k + 1) piv[(k + 1) & 1] = R(1) / nv[q];
+      }
     }
     __syncthreads();  // every read of this pivot's step is done
-    for (int t = 0; t < kPer; t++)
-      if (ei[t] >= 0) M[ei[t] * n + ej[t]] = nv[t];
+    if (j < n) {
+#pragma unroll
+      for (int q = 0; q < kPer; q++)
+        if (i0 + 16 * q < n) M[(i0 + 16 * q) * n + j] = nv[q];
+    }
     __syncthreads();  // the step's writes (and the next reciprocal) are visible
   }
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    const int i = e / n, j = e % n;
-    inv[e] = R(0.5) * (M[i * n + j] + M[j * n + i]);
+    const int i = e / n, jj = e % n;
+    inv[e] = R(0.5) * (M[i * n + jj] + M[jj * n + i]);
   }
+}
+
+// The levels of at most kBuildCells cells and (direct) the coarsest inverse, one block per
+// domain with block barriers between the levels: as launches each costs 2-3 us for less than
+// a microsecond of work (a 2000-cell column: 21 launches, now 2).
+template <typename R>
+__global__ void __launch_bounds__(kBuildThreads, 1) k_build_small(const CgDom* __restrict__ CG, int direct) {
+  MDBS_DEPENDENT_ENTRY();
+  const CgDom& G = CG[blockIdx.x];
+  const Level<R>* L = levels_of<R>(G);
+  const int nlev = G.nlev;
+  for (int l = 1; l < nlev; l++) {
+    if (L[l].cells > kBuildCells) continue;
+    for (int c = (int)threadIdx.x; c < (int)L[l].cells; c += kBuildThreads) b_coarsen(L[l - 1], L[l], c);
+    __syncthreads();
+  }
+  if (direct) coarse_inverse(L[nlev - 1], coarse_inverse_of<R>(G));
 }
 
 // ------------------------------------------------------------------ small grids in a cluster
@@ -2331,11 +2360,10 @@ void pressure_view(const PressureSolver* ps, const Fld& F, int tail_cells, CgDom
 // ------------------------------------------------------------------ batched host sequencing
 template <typename R>
 static void build_hierarchy(const BatchPlan& B, bool direct, cudaStream_t s) {
-  for (int l = 1; l < B.max_levels; l++) {
-    MDBS_LAUNCH(K_COARSEN, grid_of(B, B.lcells[l]), kBlock, s, k_coarsen<R>, B.cg, B.lcells[l], l);
-    MDBS_LAUNCH(K_DIAG, grid_of(B, B.lcells[l]), kBlock, s, k_diag<R>, B.cg, B.lcells[l], l);
-  }
-  if (direct) MDBS_LAUNCH(K_COARSEN, B.ndom, 1024, s, k_coarse_inverse<R>, B.cg);
+  for (int l = 1; l < B.max_levels; l++)
+    if (B.lcells[l].total > 0)
+      MDBS_LAUNCH(K_COARSEN, grid_of(B, B.lcells[l]), kBlock, s, k_coarsen<R>, B.cg, B.lcells[l], l);
+  MDBS_LAUNCH(K_COARSEN, B.ndom, kBuildThreads, s, k_build_small<R>, B.cg, direct ? 1 : 0);
 }
 
 // The operator depends on a_P alone, which the correctors of one step share:
@@ -2343,18 +2371,17 @@ static void build_hierarchy(const BatchPlan& B, bool direct, cudaStream_t s) {
 // hierarchy (and the coarsest inverse); each corrector then assembles only its
 // right-hand side from its HbyA.
 void launch_pressure_matrix(const BatchPlan& B, int coarse_sweeps, cudaStream_t s) {
-  MDBS_LAUNCH(K_ASSEMBLE, grid_of(B, B.cells), kBlock, s, k_assemble, B.sd, B.cells, (int)kAsmMatrix);
-  MDBS_LAUNCH(K_DIAG, grid_of(B, B.cells), kBlock, s, k_diag<double>, B.cg, B.cells, 0);
   if (!B.flexible) {
+    MDBS_LAUNCH(K_ASSEMBLE, grid_of(B, B.cells), kBlock, s, k_operator<false>, B.sd, B.cg, B.cells);
     build_hierarchy<double>(B, coarse_sweeps == 0, s);
   } else {
-    MDBS_LAUNCH(K_CONVERT, grid_of(B, B.cells), kBlock, s, k_level0_to_float, B.cg, B.cells);
+    MDBS_LAUNCH(K_ASSEMBLE, grid_of(B, B.cells), kBlock, s, k_operator<true>, B.sd, B.cg, B.cells);
     build_hierarchy<float>(B, coarse_sweeps == 0, s);
   }
 }
 
 void launch_pressure_rhs(const BatchPlan& B, cudaStream_t s) {
-  MDBS_LAUNCH(K_ASSEMBLE, grid_of(B, B.cells), kBlock, s, k_assemble, B.sd, B.cells, (int)kAsmRhs);
+  MDBS_LAUNCH(K_ASSEMBLE, grid_of(B, B.cells), kBlock, s, k_rhs, B.sd, B.cells);
 }
 
 // Traversal direction of the next kernel over each level; flips at every launch

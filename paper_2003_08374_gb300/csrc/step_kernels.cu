@@ -200,8 +200,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_alpha_flux(const StepDom* __restr
     const StepDom& S = D[dm];
     const int lb = b - w.blk[dm];
     double v = 0.0;
-    for (int r = 0; r < w.rep; r++) {
-      const long long t = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
+    for (int r = 0; r < S.rep; r++) {
+      const long long t = ((long long)lb * S.rep + r) * blockDim.x + threadIdx.x;
       if (t < total_faces(S.P)) v += b_alpha_flux(S.P, S.F, t);
     }
     const double sum = block_sum(v);
@@ -712,8 +712,8 @@ __global__ void k_field_stats(const StepDom* __restrict__ D, Work w) {
     const StepDom& S = D[dm];
     const int lb = b - w.blk[dm];
     double mass = 0.0, amin = INFINITY, amax = -INFINITY, bad = 0.0;
-    for (int r = 0; r < w.rep; r++) {
-      const long long c = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
+    for (int r = 0; r < S.rep; r++) {
+      const long long c = ((long long)lb * S.rep + r) * blockDim.x + threadIdx.x;
       if (c < S.P.cells) {
         const double a = S.F.alpha[c];
         mass += S.F.phi[c] * a * S.P.V;
@@ -782,8 +782,8 @@ __global__ void k_cfl(const StepDom* __restrict__ D, Work w) {
     const StepDom& S = D[dm];
     const int lb = b - w.blk[dm];
     double vmax = 0.0;
-    for (int r = 0; r < w.rep; r++) {
-      const long long t = ((long long)lb * w.rep + r) * blockDim.x + threadIdx.x;
+    for (int r = 0; r < S.rep; r++) {
+      const long long t = ((long long)lb * S.rep + r) * blockDim.x + threadIdx.x;
       int d, i, j, k;
       long long f;
       if (decode_face(S.P, t, d, i, j, k, f)) {
