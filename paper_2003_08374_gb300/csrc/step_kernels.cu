@@ -163,10 +163,14 @@ __device__ __forceinline__ double b_alpha_flux(const Prm& P, const Fld& F, long 
           double gf[3] = {0.0, 0.0, 0.0};
           for (int e = 0; e < P.dim; e++)
             gf[e] = 0.5 * (cgrad(F.alpha, P, e, i - di, j - dj, k - dk) + cgrad(F.alpha, P, e, i, j, k));
-          const double mag = sqrt(gf[0] * gf[0] + gf[1] * gf[1] + gf[2] * gf[2]);
-          const double nfc = gf[d] / (mag + 1e-8 * inv_h);
-          const double w = P.c_alpha * fabs(uf) * nfc * P.A;
-          rel = ge0z(w) ? w * al * (1.0 - ar) : w * ar * (1.0 - al);
+          // gf[d] = 0 (most faces of a tank: the air holds no liquid at all) has no
+          // compression flux; the root and the division are a quarter of a face's FP64 work
+          if (nz(gf[d])) {
+            const double mag = sqrt(gf[0] * gf[0] + gf[1] * gf[1] + gf[2] * gf[2]);
+            const double nfc = gf[d] / (mag + 1e-8 * inv_h);
+            const double w = P.c_alpha * fabs(uf) * nfc * P.A;
+            rel = ge0z(w) ? w * al * (1.0 - ar) : w * ar * (1.0 - al);
+          }
         }
         hi = Q * van_leer(aU, aD, aUU) + rel;
       }
@@ -393,9 +397,13 @@ __device__ __forceinline__ void b_normals(const Prm& P, const Fld& F, long long 
   decode_cell(P, c, i, j, k);
   double g[3] = {0.0, 0.0, 0.0};
   for (int e = 0; e < P.dim; e++) g[e] = fluid_grad(F.alpha, P, F, e, i, j, k, c);
-  const double mag = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-  const double inv_den = 1.0 / (mag + P.reg_m);
-  double m[3] = {g[0] * inv_den, g[1] * inv_den, g[2] * inv_den};
+  // a zero gradient has a zero normal, without the root and the division
+  double m[3] = {0.0, 0.0, 0.0};
+  if (nz(g[0]) || nz(g[1]) || nz(g[2])) {
+    const double mag = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+    const double inv_den = 1.0 / (mag + P.reg_m);
+    for (int e = 0; e < 3; e++) m[e] = g[e] * inv_den;
+  }
   const double nw[3] = {F.nw[0][c], F.nw[1][c], F.nw[2][c]};
   if (nw[0] != 0.0 || nw[1] != 0.0 || nw[2] != 0.0) {
     const double mm = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
