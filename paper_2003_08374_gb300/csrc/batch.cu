@@ -143,6 +143,8 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
   if (e == cudaSuccess) e = cudaMemcpy(B.cg, cg, ndom * sizeof(CgDom), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&B.any_flag, 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(B.any_flag, 0, 2 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&B.act, ndom * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(B.act, 0, ndom * sizeof(int));
   std::vector<CgVec> cv(ndom);
   for (int d = 0; d < ndom; d++) {
     const Prm& P = sd[d].P;
@@ -173,6 +175,7 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
     w.ndom = ndom;
     w.total = totals[space];
     w.rep = reps[space];
+    w.act = B.act;
     return w;
   };
   B.cells = work(0);
@@ -200,6 +203,8 @@ void plan_destroy(BatchPlan* B) {
   if (B->table_storage) cudaFree(B->table_storage);
   if (B->sd) cudaFree(B->sd);
   if (B->cg) cudaFree(B->cg);
+  if (B->act) cudaFree(B->act);
+  B->act = nullptr;
   if (B->cv) cudaFree(B->cv);
   delete B->one_cg;
   B->cv = nullptr;

@@ -125,19 +125,25 @@ struct Work {
   int ndom;
   int total;       // work items; item i of a domain covers elements [i*rep*blockDim, (i+1)*rep*blockDim)
   int rep;         // blockDim-sized rows per work item
+  int* act;        // device: per domain, whether its CG still iterates
 };
 
-// domain owning flat block b: the largest d with blk[d] <= b (empty domains are skipped)
+// domain owning flat block b: the largest d with blk[d] <= b (empty domains are skipped).
+// Called by whole warps with the same b: the last step looks at 32 entries at once (a
+// binary search over 16 domains was four dependent loads ahead of every item's work).
 __device__ __forceinline__ int work_domain(const Work& w, int b) {
-  int lo = 0, hi = w.ndom - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
+  if (w.ndom == 1) return 0;
+  int lo = 0, hi = w.ndom;  // the answer lies in [lo, hi)
+  while (hi - lo > 32) {
+    const int mid = (lo + hi) >> 1;
     if (w.blk[mid] <= b)
       lo = mid;
     else
-      hi = mid - 1;
+      hi = mid;
   }
-  return lo;
+  const int d = lo + (int)(threadIdx.x & 31u);
+  const unsigned m = __ballot_sync(0xffffffffu, d < hi && w.blk[d] <= b);
+  return lo + 31 - __clz((int)m);
 }
 
 // per-domain view of the step kernels
@@ -326,7 +332,7 @@ struct BatchPlan {
   int ndom;
   int grid_cap;               // persistent grid: SMs x resident blocks
   Work cells, faces, dom;     // per-domain cells, faces (one row per item), one block per domain
-  Work rcells, rfaces;        // the same with kRepBig rows per item: kernels with block reductions
+  Work rcells, rfaces;        // the same with StepDom::rep rows per item: kernels with block reductions
   Work cgcells;               // CG vectors: kRepBig rows per item, domains solved by clusters left out
   int n_small, n_big;         // domains whose CG solve runs in a cluster, and the others
   const int *small_idx, *big_idx;  // device: their indexes
@@ -360,6 +366,7 @@ struct BatchPlan {
   CgDom* one_cg;              // host copies, for kernels over a single domain (ndom == 1)
   CgVec one_cv;
   int* table_storage;         // device memory of every block table
+  int* act;                   // device: per domain, whether its CG still iterates
   int* any_flag;              // device: some domain still iterating (CG WHILE condition); [1] arrivals
   int* err_flag;              // device: a kernel's bounded wait ran out (the batch's results are invalid)
 };

@@ -426,12 +426,12 @@ __device__ __forceinline__ void smooth_item(const CgDom& G, int l, int lb, unsig
 }
 
 template <typename R, int REP, bool PRO = false>
-__global__ void __launch_bounds__(kBlock, REP == 1 ? 8 : 1)
+__global__ void __launch_bounds__(kBlock)
     k_smooth(const CgDom* __restrict__ C, Work w, int l, int col, int zero, int rev) {
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK_DIR(w, rev)
     const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
+    if (w.act[dm] == 0) continue;
     smooth_item<R, REP, PRO>(G, l, lb, threadIdx.x, col, zero);
   }
 }
@@ -445,19 +445,25 @@ struct LvPair {
 // The half sweep with one cell a thread.  Everything static -- the cell's position, its six
 // coefficients, its reciprocal diagonal -- is in registers before the wait on the preceding
 // kernel, so what remains after it is one round of loads, the fma chain and the store; a
-// kernel's successors fetch their coefficients while its last blocks finish.  For a single
-// domain: its levels are passed by value (their pointers are in the constant bank), and the
-// loop it runs in is its own (no flag to test).  A batch keeps k_smooth, whose blocks leave
-// a converged domain before they load anything: prefetching made its fine sweeps 45 us
-// where k_smooth takes 34 (16 uneven domains, 4.7 M cells).
-template <typename R, bool PRO>
-__global__ void __launch_bounds__(kBlock, PRO && sizeof(R) == 8 ? 4 : 5)
-    k_sweep(const __grid_constant__ LvPair<R> one, int items, int col, int zero, int rev) {
+// kernel's successors fetch their coefficients while its last blocks finish.  ONE: a single
+// domain, its levels passed by value (their pointers are in the constant bank), in a loop of
+// its own (no flag to test).  A batch's blocks wait first and leave a converged domain before
+// they load anything.  CTAs an SM: the plain sweep as many as its registers allow without
+// spills (16.8 M cells FP32 66 -> 59 us, FP64 107 -> 103 against 5), the one that adds the
+// correction fewer (FP32 8 instead of 5: 78 -> 103 us).
+template <typename R, bool PRO, bool ONE>
+__global__ void __launch_bounds__(kBlock, PRO ? (sizeof(R) == 8 ? 4 : 5) : (sizeof(R) == 8 ? 6 : 8))
+    k_sweep(const __grid_constant__ LvPair<R> one, const CgDom* __restrict__ C, Work w, int l, int col, int zero,
+            int rev) {
   MDBS_PDL_TRIGGER();
-  const Level<R>& L = one.fine;
-  bool waited = false;
-  for (int i_ = blockIdx.x; i_ < items; i_ += gridDim.x) {
-    const int lb = rev ? items - 1 - i_ : i_;
+  bool waited = !ONE;
+  if (!ONE) MDBS_PDL_WAIT();
+  for (int i_ = blockIdx.x; i_ < w.total; i_ += gridDim.x) {
+    const int b_ = rev ? w.total - 1 - i_ : i_;
+    const int dm = ONE ? 0 : work_domain(w, b_);
+    if (!ONE && w.act[dm] == 0) continue;
+    const int lb = ONE ? b_ : b_ - w.blk[dm];
+    const Level<R>& L = ONE ? one.fine : levels_of<R>(C[dm])[l];
     const int n0 = L.n[0], n1 = L.n[1], n2 = L.n[2];
     const unsigned half = (unsigned)(n0 + 1) >> 1, total = half * (unsigned)n1 * (unsigned)n2;
     const unsigned t = (unsigned)lb * kBlock + threadIdx.x;
@@ -499,7 +505,7 @@ __global__ void __launch_bounds__(kBlock, PRO && sizeof(R) == 8 ? 4 : 5)
       if (zp) x5 = x[c + sz];
       if constexpr (PRO) {
         // the neighbours' corrections (see smooth_cell_corr)
-        const Level<R>& Co = one.coarse;
+        const Level<R>& Co = ONE ? one.coarse : levels_of<R>(C[dm])[l + 1];
         const R* __restrict__ ex = Co.x;
         const int a = Co.cz[0], b = Co.cz[1], d = Co.cz[2];
         const unsigned m0 = (unsigned)Co.n[0], m01 = m0 * (unsigned)Co.n[1], he = (m0 + 1) >> 1;
@@ -587,7 +593,7 @@ __global__ void __launch_bounds__(kBlock, 3)
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK_DIR(w, rev)
     const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
+    if (w.act[dm] == 0) continue;
     const Level<R>& Lr = levels_of<R>(G)[l];
     const int n0 = Lr.n[0], n1 = Lr.n[1], n2 = Lr.n[2];
     const unsigned half = (unsigned)n0 >> 1;  // both runs: n0 is a multiple of 2 V
@@ -984,7 +990,7 @@ __global__ void k_zero(const CgDom* __restrict__ C, Work w, int l, int rev, int 
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK_DIR(w, rev)
     const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
+    if (w.act[dm] == 0) continue;
     const Level<R>& L = levels_of<R>(G)[l];
     R* __restrict__ x = sel ? L.x2 : L.x;
     for (int r = 0; r < w.rep; r++) {
@@ -1032,8 +1038,9 @@ __device__ __forceinline__ void b_resid_restrict(const Level<R>& Fi, const Level
 // of a coarse level: 20 us for a level of 16^3, however small (cold, ncu).
 constexpr int kRestCells = 64;
 
+// 5 CTAs an SM (4 in parentheses): 128^3 FP64 28.0 us (30.7), 512 x 128 x 256 FP32 101 (118)
 template <typename R, bool ONE>
-__global__ void __launch_bounds__(kBlock, 4)
+__global__ void __launch_bounds__(kBlock, 5)
     k_resid_restrict(const __grid_constant__ LvPair<R> one, const CgDom* __restrict__ C, Work w, int l, int rev,
                      int sel, int mask, int fold) {
   static_assert(kBlock == 4 * kRestCells, "four threads a coarse cell");
@@ -1049,7 +1056,7 @@ __global__ void __launch_bounds__(kBlock, 4)
     const int b_ = rev ? w.total - 1 - i_ : i_;
     const int dm = ONE ? 0 : work_domain(w, b_);
     const int lb = ONE ? b_ : b_ - w.blk[dm];
-    if (!ONE && C[dm].scal[kCond] == 0.0) continue;
+    if (!ONE && w.act[dm] == 0) continue;
     const Level<R>& Fi = ONE ? one.fine : levels_of<R>(C[dm])[l];
     const Level<R>& Co = ONE ? one.coarse : levels_of<R>(C[dm])[l + 1];
     const long long ci = (long long)lb * kRestCells + t;
@@ -1133,7 +1140,7 @@ __global__ void k_prolong(const CgDom* __restrict__ C, Work w, int l, int rev, i
   MDBS_DEPENDENT_ENTRY();
   FOR_WORK_DIR(w, rev)
     const CgDom& G = C[dm];
-    if (G.scal[kCond] == 0.0) continue;
+    if (w.act[dm] == 0) continue;
     const Level<R>* L = levels_of<R>(G);
     Level<R> Fi = L[l];
     if (sel) Fi.x = Fi.x2;
@@ -1625,19 +1632,24 @@ __device__ __forceinline__ double apply_A0(const Fld& F, const Prm& P, const dou
 // CTAs that send their factors to one of them: 2.72 ms.  Above kMidItems the arrivals cost
 // more than the launch saves.)
 constexpr int kMidItems = 256;  // a block of kBlock threads then folds a partial sum a thread
+// Rows whose loads are in flight together (row by row, each row's loads waited for the stores
+// of the row before).  k_update_xr, 2.1 M / 16.8 M cells: row by row 28.8 / 170 us, 2 rows
+// 23.7 / 151, 4 rows 20.8 / 154, 8 rows 26.5 / 185 (registers).
+constexpr int kGroup = 4;
 enum { kBatch = 0, kPlain = 1, kLarge = kRepBig };
 
 // One block's loop over its items: V the domain, lb the index of the partial sum, kRows
 // rows from cell c0 (+ the thread) on.
 #define CG_ITEMS(ITEMS, BLK, REV)                                                                \
   constexpr int kRows = FORM == kPlain ? 1 : kRepBig;                                            \
+  constexpr int kG = kRows < kGroup ? kRows : kGroup;                                            \
   for (int i_ = blockIdx.x; i_ < (ITEMS); i_ += gridDim.x) {                                     \
     const int b_ = (REV) ? (ITEMS) - 1 - i_ : i_;                                                \
     const int dm = FORM != kBatch ? 0 : work_domain((BLK), b_);                                  \
     const int lb = FORM != kBatch ? b_ : b_ - (BLK).blk[dm];                                     \
     const CgVec& V = FORM != kBatch ? one : table[dm];                                           \
     const unsigned c0 = (unsigned)lb * (unsigned)kRows * kBlock + threadIdx.x;
-#define CG_ACTIVE() (FORM != kBatch || V.scal[kCond] != 0.0)
+#define CG_ACTIVE(BLK) (FORM != kBatch || (BLK).act[dm] != 0)
 
 __device__ __forceinline__ void cg_sum(double s, double* out) {
   s = block_sum(s);
@@ -1714,7 +1726,7 @@ __global__ void __launch_bounds__(kBlock, 4)
   MDBS_PDL_TRIGGER();
   MDBS_PDL_WAIT();
   CG_ITEMS(items, w, rev)
-    if (!CG_ACTIVE()) continue;
+    if (!CG_ACTIVE(w)) continue;
     double s = 0.0;
 #pragma unroll 2
     for (int r = 0; r < kRows; r++) {
@@ -1737,7 +1749,7 @@ __global__ void k_update_xr(const __grid_constant__ CgVec one, const CgVec* __re
   MDBS_PDL_TRIGGER();
   MDBS_PDL_WAIT();
   CG_ITEMS(items, w, rev)
-    if (!CG_ACTIVE()) continue;
+    if (!CG_ACTIVE(w)) continue;
     const double al = V.scal[kAlpha];
     const unsigned n = V.cells, n0 = (unsigned)V.n[0], he = (n0 + 1) >> 1;
     double* __restrict__ p = V.p;
@@ -1746,17 +1758,29 @@ __global__ void k_update_xr(const __grid_constant__ CgVec one, const CgVec* __re
     const double* __restrict__ qv = V.q;
     double s = 0.0;
 #pragma unroll
-    for (int r = 0; r < kRows; r++) {
-      const unsigned c = c0 + (unsigned)r * kBlock;
-      if (c < n) {
-        // p is in natural order: the cell at x-split position c
+    for (int r0 = 0; r0 < kRows; r0 += kG) {
+      double pv[kG], dd[kG], rc[kG], qc[kG];
+#pragma unroll
+      for (int g = 0; g < kG; g++) {
+        const unsigned c = min(c0 + (unsigned)(r0 + g) * kBlock, n - 1u);
+        // p is in natural order and the vectors are not: the thread takes p's cell c, with d
+        // from that cell's position (a warp reads two runs of d), and r's position c
         const unsigned row = fastdiv(c, V.dn0), x = c - row * n0;
-        double* const pc = p + (row * n0 + (x < he ? 2 * x : 2 * (x - he) + 1));
-        *pc = fma(al, dv[c], *pc);
-        const double rc = fma(-al, qv[c], rv[c]);
-        rv[c] = rc;
-        if (narrow) V.bf[c] = (float)rc;  // the next FP32 V-cycle's right-hand side
-        s = fma(rc, rc, s);
+        pv[g] = p[c];
+        dd[g] = dv[row * n0 + (x >> 1) + ((x & 1) ? he : 0)];
+        rc[g] = rv[c];
+        qc[g] = qv[c];
+      }
+#pragma unroll
+      for (int g = 0; g < kG; g++) {
+        const unsigned c = c0 + (unsigned)(r0 + g) * kBlock;
+        if (c < n) {
+          p[c] = fma(al, dd[g], pv[g]);
+          const double v = fma(-al, qc[g], rc[g]);
+          rv[c] = v;
+          if (narrow) V.bf[c] = (float)v;  // the next FP32 V-cycle's right-hand side
+          s = fma(v, v, s);
+        }
       }
     }
     if (FORM != kPlain) cg_sum(s, V.partials + lb);
@@ -1764,14 +1788,15 @@ __global__ void k_update_xr(const __grid_constant__ CgVec one, const CgVec* __re
 }
 
 // partial r.z and (FLEX) z.q; in flexible CG z is the FP32 V-cycle's result, widened here
-// (no separate pass)
+// (no separate pass; widening it again in k_update_d instead of storing it is slower: 10.9 ->
+// 13.9 us there, 2.1 M cells, the conversions run on the FP64 pipe)
 template <int FORM, bool FLEX>
 __global__ void k_dots_rz(const __grid_constant__ CgVec one, const CgVec* __restrict__ table, Work w, int items,
                           int rev) {
   MDBS_PDL_TRIGGER();
   MDBS_PDL_WAIT();
   CG_ITEMS(items, w, rev)
-    if (!CG_ACTIVE()) continue;
+    if (!CG_ACTIVE(w)) continue;
     const unsigned n = V.cells;
     const double* __restrict__ rv = V.r;
     double* __restrict__ z = V.z;
@@ -1779,18 +1804,31 @@ __global__ void k_dots_rz(const __grid_constant__ CgVec one, const CgVec* __rest
     const float* __restrict__ zf = V.xf;
     double rz = 0.0, zq = 0.0;
 #pragma unroll
-    for (int r = 0; r < kRows; r++) {
-      const unsigned c = c0 + (unsigned)r * kBlock;
-      if (c < n) {
-        double zc;
+    for (int r0 = 0; r0 < kRows; r0 += kG) {
+      double rc[kG], zc[kG], qc[kG];
+      float zs[kG];
+#pragma unroll
+      for (int g = 0; g < kG; g++) {
+        const unsigned c = min(c0 + (unsigned)(r0 + g) * kBlock, n - 1u);
+        rc[g] = rv[c];
         if (FLEX) {
-          zc = (double)zf[c];
-          z[c] = zc;
+          zs[g] = zf[c];
+          qc[g] = qv[c];
         } else {
-          zc = z[c];
+          zc[g] = z[c];
         }
-        rz = fma(rv[c], zc, rz);
-        if (FLEX) zq = fma(zc, qv[c], zq);
+      }
+#pragma unroll
+      for (int g = 0; g < kG; g++) {
+        const unsigned c = c0 + (unsigned)(r0 + g) * kBlock;
+        if (c < n) {
+          if (FLEX) {
+            zc[g] = (double)zs[g];
+            z[c] = zc[g];
+          }
+          rz = fma(rc[g], zc[g], rz);
+          if (FLEX) zq = fma(zc[g], qc[g], zq);
+        }
       }
     }
     cg_sum(rz, V.partials + lb);
@@ -1805,7 +1843,7 @@ __global__ void k_update_d(const __grid_constant__ CgVec one, const CgVec* __res
   MDBS_PDL_TRIGGER();
   MDBS_PDL_WAIT();
   CG_ITEMS(items, w, rev)
-    if (!CG_ACTIVE()) continue;
+    if (!CG_ACTIVE(w)) continue;
     const bool first = V.scal[kIt] == 0.0;
     const double be = V.scal[kBeta];
     const unsigned n = V.cells;
@@ -1862,7 +1900,10 @@ __global__ void k_finalize(const CgDom* __restrict__ C, Work w, int mode, int tw
     }
     a = block_sum(a);
     if (two) b = block_sum(b);
-    if (threadIdx.x == 0) cg_scalars(scal, mode, two, a, b, tol, max_it);
+    if (threadIdx.x == 0) {
+      cg_scalars(scal, mode, two, a, b, tol, max_it);
+      if (mode == 0 || mode == 2) w.act[blockIdx.x] = scal[kCond] != 0.0;
+    }
   }
   if (mode == 1 || mode == 3) return;
   __shared__ int s_last;
@@ -1887,7 +1928,8 @@ __global__ void k_finalize(const CgDom* __restrict__ C, Work w, int mode, int tw
 // mode 1: d.q; mode 2: r.r; mode 3: r.z and (FLEX) z.q, z widened from the FP32 V-cycle.
 template <int MODE, bool FLEX>
 __global__ void __launch_bounds__(kBlock)
-    k_sum_final(const __grid_constant__ CgVec V, double tol, int max_it, int* flag, cudaGraphConditionalHandle handle,
+    k_sum_final(const __grid_constant__ CgVec V, double tol, int max_it, int* flag, int* act,
+                cudaGraphConditionalHandle handle,
                 int use_handle) {
   MDBS_PDL_TRIGGER();
   MDBS_PDL_WAIT();
@@ -1942,6 +1984,7 @@ __global__ void __launch_bounds__(kBlock)
   if (MODE == 2) {
     const int any = V.scal[kCond] != 0.0;
     flag[0] = any;
+    act[0] = any;
     if (use_handle) cudaGraphSetConditional(handle, any ? 1u : 0u);
   }
 }
@@ -2427,9 +2470,9 @@ static void smooth_half_t(const BatchPlan& B, int l, int col, int zero, Dirs& D,
     case 2: MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_smooth<R, 2, PRO>), B.cg, w, l, col, zero, rev); break;
     default:
       if (B.one_cg)
-        MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_sweep<R, PRO>), level_pair<R>(B, l), w.total, col, zero, rev);
+        MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_sweep<R, PRO, true>), level_pair<R>(B, l), B.cg, w, l, col, zero, rev);
       else
-        MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_smooth<R, 1, PRO>), B.cg, w, l, col, zero, rev);
+        MDBS_LAUNCH(id, grid_of(B, w), kBlock, s, (k_sweep<R, PRO, false>), LvPair<R>{}, B.cg, w, l, col, zero, rev);
   }
 }
 
@@ -2653,7 +2696,7 @@ cudaError_t pressure_solve(const BatchPlan& B, double tol, int max_it, int nu1, 
     if (B.ndom == 1 && w.total <= kMidItems) {
       const int rows = (int)((B.one_cv.cells + kBlock - 1) / kBlock);
       auto sums = [&](int id, auto kernel) {
-        MDBS_LAUNCH(id, w.total, kBlock, bs, kernel, B.one_cv, tol, max_it, B.any_flag, handle, use);
+        MDBS_LAUNCH(id, w.total, kBlock, bs, kernel, B.one_cv, tol, max_it, B.any_flag, B.act, handle, use);
       };
       sums(K_DOTS, flexible ? k_sum_final<3, true> : k_sum_final<3, false>);
       MDBS_LAUNCH(K_UPDATE_D, rows, kBlock, bs, (k_update_d<kPlain>), B.one_cv, B.cv, w, rows, D.next(0));
