@@ -885,22 +885,30 @@ int mdbs_set_fields(mdbs_sim* s, const double* alpha, const double* ux, const do
   // transport through a velocity field divergence-free only to the pressure tolerance
   // moves alpha outside [0, 1] by dt |div(A u)| / (phi V) per step, so the range also
   // admits the extremes its own steps have reached.
-  // The check runs on the device: alpha goes to the low-order saturation scratch (which
-  // the next step overwrites), a kernel flags any value out of range, and only an
-  // accepted field is copied into place, so a rejected call leaves the state unchanged.
+  // alpha goes to the low-order saturation scratch (which the next step overwrites), and only
+  // an accepted field is copied into place, so a rejected call leaves the state unchanged.
+  // The check runs on the device, where a kernel flags any value out of range, except for
+  // small fields: up to kHostCheck cells the caller's array is read here (16384 cells, 5 us),
+  // which the kernel, the flag's way back and the wait (30 us) cannot match.
+  constexpr long long kHostCheck = 16384;
   const double lo = std::min(-1e-9, s->alpha_lo_seen), hi = std::max(1.0 + 1e-9, s->alpha_hi_seen);
   double* stage = s->F.aL;
   CK(cudaMemcpyAsync(stage, alpha, s->P.cells * 8, cudaMemcpyHostToDevice, s->stream));
-  CK(cudaMemsetAsync(s->scal + kSlotCheck, 0, sizeof(double), s->stream));
-  {
+  bool bad = false;
+  if (s->P.cells <= kHostCheck) {
+    for (long long c = 0; c < s->P.cells; c++) bad |= !(alpha[c] >= lo && alpha[c] <= hi);
+    if (bad) CK(cudaStreamSynchronize(s->stream));  // the copy has left the caller's array
+  } else {
+    CK(cudaMemsetAsync(s->scal + kSlotCheck, 0, sizeof(double), s->stream));
     const long long blocks = std::min<long long>((s->P.cells + 255) / 256, 4096);
     k_check_range<<<(unsigned)blocks, 256, 0, s->stream>>>(stage, s->P.cells, lo, hi, s->scal + kSlotCheck);
     CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(s->host_scal + kSlotCheck, s->scal + kSlotCheck, sizeof(double), cudaMemcpyDeviceToHost,
+                       s->stream));
+    CK(cudaStreamSynchronize(s->stream));
+    bad = s->host_scal[kSlotCheck] != 0.0;
   }
-  CK(cudaMemcpyAsync(s->host_scal + kSlotCheck, s->scal + kSlotCheck, sizeof(double), cudaMemcpyDeviceToHost,
-                     s->stream));
-  CK(cudaStreamSynchronize(s->stream));
-  if (s->host_scal[kSlotCheck] != 0.0)
+  if (bad)
     return fail(s, MDBS_ERR_ARG,
                 "alpha must lie in [0, 1] (to 1e-9, or within the extremes this simulation reached)");
   const double* src[3] = {ux, uy, uz};
