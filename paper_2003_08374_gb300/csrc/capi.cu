@@ -888,8 +888,9 @@ int mdbs_set_fields(mdbs_sim* s, const double* alpha, const double* ux, const do
   // alpha goes to the low-order saturation scratch (which the next step overwrites), and only
   // an accepted field is copied into place, so a rejected call leaves the state unchanged.
   // The check runs on the device, where a kernel flags any value out of range, except for
-  // small fields: up to kHostCheck cells the caller's array is read here (16384 cells, 5 us),
-  // which the kernel, the flag's way back and the wait (30 us) cannot match.
+  // small fields: up to kHostCheck cells the caller's array is read here, without the kernel,
+  // the flag's way back and a wait (the whole call, device -> host check: 2000 cells 88 ->
+  // 66 us, 8192 126 -> 98, 16384 121 -> 116, where the reading costs what the wait does).
   constexpr long long kHostCheck = 16384;
   const double lo = std::min(-1e-9, s->alpha_lo_seen), hi = std::max(1.0 + 1e-9, s->alpha_hi_seen);
   double* stage = s->F.aL;
