@@ -291,7 +291,7 @@ def peaks():
 
 
 def kernel_source_hash():
-    """Hash of the half-sweep kernel's source (smooth_cell, smooth_cell_corr, k_smooth)."""
+    """Hash of the half-sweep kernels' source (smooth_cell, smooth_cell_corr, k_smooth, k_sweep)."""
     src = open(os.path.join(ROOT, "paper_2003_08374_gb300", "csrc", "pressure.cu")).read()
     a = src.index("// One red-black Gauss-Seidel update of cell c")
     b = src.index("// ------------------------------------------------------------------ fused red-black sweep (FP32)")
