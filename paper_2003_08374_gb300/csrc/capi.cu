@@ -887,16 +887,24 @@ int mdbs_set_fields(mdbs_sim* s, const double* alpha, const double* ux, const do
   // admits the extremes its own steps have reached.
   // alpha goes to the low-order saturation scratch (which the next step overwrites), and only
   // an accepted field is copied into place, so a rejected call leaves the state unchanged.
-  // The check runs on the device, where a kernel flags any value out of range, except for
-  // small fields: up to kHostCheck cells the caller's array is read here, without the kernel,
-  // the flag's way back and a wait (the whole call, device -> host check: 2000 cells 88 ->
-  // 66 us, 8192 126 -> 98, 16384 121 -> 116, where the reading costs what the wait does).
+  // The check runs on the device, in the order of the stream, where a kernel flags any value
+  // out of range, except for small fields in pageable memory: up to kHostCheck cells that
+  // array is read here, without the kernel, the flag's way back and a wait.  The copy below
+  // reads pageable memory when it is called; memory the runtime knows (pinned, managed) may
+  // be filled by work queued ahead of the copy, so its values are not yet there to be read.
+  // (The whole call, device -> host check: 2000 cells 88 -> 66 us, 8192 126 -> 98, 16384
+  // 121 -> 116, where the reading costs what the wait does.)
   constexpr long long kHostCheck = 16384;
   const double lo = std::min(-1e-9, s->alpha_lo_seen), hi = std::max(1.0 + 1e-9, s->alpha_hi_seen);
   double* stage = s->F.aL;
   CK(cudaMemcpyAsync(stage, alpha, s->P.cells * 8, cudaMemcpyHostToDevice, s->stream));
-  bool bad = false;
+  bool bad = false, host = false;
   if (s->P.cells <= kHostCheck) {
+    cudaPointerAttributes at;
+    CK(cudaPointerGetAttributes(&at, alpha));
+    host = at.type == cudaMemoryTypeUnregistered;
+  }
+  if (host) {
     for (long long c = 0; c < s->P.cells; c++) bad |= !(alpha[c] >= lo && alpha[c] <= hi);
     if (bad) CK(cudaStreamSynchronize(s->stream));  // the copy has left the caller's array
   } else {
