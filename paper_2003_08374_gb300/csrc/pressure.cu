@@ -1910,6 +1910,7 @@ __global__ void k_finalize(const CgDom* __restrict__ C, Work w, int mode, int tw
   if (threadIdx.x == 0) {
     __threadfence();
     s_last = gridDim.x == 1 || atomicAdd(flag + 1, 1) == (int)gridDim.x - 1;
+    __threadfence();  // the arrivals before the conditions they announce
   }
   __syncthreads();
   if (!s_last) return;
