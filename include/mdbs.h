@@ -358,6 +358,13 @@ int mdbs_profile_read(const mdbs_sim* sim, int32_t id, const char** name, double
 int64_t mdbs_debug_array(const mdbs_sim* sim, const char* name, double* out, int64_t capacity);
 
 /*
+ * Test aid: plans this simulation (and a batch it joins afterwards) as on a device that
+ * cannot run thread-block clusters of more than max_ctas CTAs (0: none at all).  Results do
+ * not depend on it.  MDBS_ERR_ARG while the simulation belongs to a batch.
+ */
+int mdbs_debug_cluster_limit(mdbs_sim* sim, int32_t max_ctas);
+
+/*
  * Self-test of the bounded device waits (no counterpart in the paper).  Kernels that
  * wait on asynchronous copies (the fused sweeps' mbarriers) give up after one second,
  * record the failure (the step then returns MDBS_ERR_CUDA) and return, so a lost

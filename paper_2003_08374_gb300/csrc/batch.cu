@@ -18,7 +18,8 @@ long long faces_total(const Prm& P) { return P.nf[0] + P.nf[1] + (P.dim == 3 ? P
 }  // namespace
 
 cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexible, int smooth_rows, int snake,
-                        int sweep_kz, int tail_ctas, int coarse_coop, int vec_sweeps, BatchPlan* out) {
+                        int sweep_kz, int tail_ctas, int coarse_coop, int vec_sweeps, int cluster_limit,
+                        BatchPlan* out) {
   BatchPlan B{};
   B.ndom = ndom;
   B.flexible = flexible;
@@ -43,14 +44,15 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
   // after the spaces: the indexes of the small domains, then of the others
   std::vector<int> tab((size_t)nspace * (ndom + 1) + ndom, 0);
   int* const idx = &tab[(size_t)nspace * (ndom + 1)];
-  for (int d = 0; d < ndom; d++)
-    if (cg[d].small) idx[B.n_small++] = d;
-  for (int d = 0; d < ndom; d++)
-    if (!cg[d].small) idx[B.n_small + B.n_big++] = d;
+  std::vector<char> small(ndom);
   {
-    cudaError_t e = plan_clusters(cg, ndom, flexible, tail_ctas, sms, &B);
+    cudaError_t e = plan_clusters(cg, ndom, flexible, tail_ctas, sms, cluster_limit, small.data(), &B);
     if (e != cudaSuccess) return e;
   }
+  for (int d = 0; d < ndom; d++)
+    if (small[d]) idx[B.n_small++] = d;
+  for (int d = 0; d < ndom; d++)
+    if (!small[d]) idx[B.n_small + B.n_big++] = d;
   auto fill = [&](int space, auto count) -> int {
     int* t = &tab[(size_t)space * (ndom + 1)];
     long long acc = 0;
@@ -73,7 +75,7 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
   totals[2] = fill(2, [&](int) { return 1LL; });
   totals[3] = fill(3, [&](int d) { return red_items(sd[d].P.cells, sd[d].rep); });
   totals[4] = fill(4, [&](int d) { return red_items(faces_total(sd[d].P), sd[d].rep); });
-  totals[scg] = fill(scg, [&](int d) { return cg[d].small ? 0LL : cg_items(sd[d].P.cells); });
+  totals[scg] = fill(scg, [&](int d) { return small[d] ? 0LL : cg_items(sd[d].P.cells); });
   B.max_first = 0;
   B.max_levels = 0;
   B.any_cfl = 0;

@@ -145,6 +145,7 @@ struct mdbs_sim {
   bool in_batch;
   std::string err;
   mdbs_tuning tun;    // schedule of the multigrid kernels
+  int cluster_limit = kClusterLimit;  // mdbs_debug_cluster_limit
   Exec ex;            // batch of one: this simulation alone
 };
 
@@ -443,10 +444,11 @@ cudaError_t record_step(Exec& ex, const mdbs_options& opt, cudaStream_t st, bool
   return le != cudaSuccess ? le : cudaGetLastError();
 }
 
-cudaError_t exec_setup(Exec& ex, const StepDom* sd, const CgDom* cg, int ndom, int flexible, const mdbs_tuning& t) {
+cudaError_t exec_setup(Exec& ex, const StepDom* sd, const CgDom* cg, int ndom, int flexible, const mdbs_tuning& t,
+                       int cluster_limit) {
   cudaError_t e =
       plan_create(sd, cg, ndom, flexible, t.smooth_rows, t.snake, t.sweep_kz, t.tail_ctas, t.coarse_coop,
-                  t.vec_sweeps, &ex.plan);
+                  t.vec_sweeps, cluster_limit, &ex.plan);
   if (e != cudaSuccess) return e;
   ex.planned = true;
   if (!ex.cap_stream) e = cudaStreamCreateWithFlags(&ex.cap_stream, cudaStreamNonBlocking);
@@ -544,7 +546,7 @@ cudaError_t sim_exec_setup(mdbs_sim* s) {
   StepDom sd = step_view(s);
   CgDom cg;
   pressure_view(s->ps, s->F, s->tun.tail_cells, &cg);
-  return exec_setup(s->ex, &sd, &cg, 1, s->precision != 0, s->tun);
+  return exec_setup(s->ex, &sd, &cg, 1, s->precision != 0, s->tun, s->cluster_limit);
 }
 
 cudaError_t batch_exec_setup(mdbs_batch* b) {
@@ -555,11 +557,13 @@ cudaError_t batch_exec_setup(mdbs_batch* b) {
   const int n = (int)b->sims.size();
   std::vector<StepDom> sd(n);
   std::vector<CgDom> cg(n);
+  int limit = kClusterLimit;
   for (int i = 0; i < n; i++) {
     sd[i] = step_view(b->sims[i]);
     pressure_view(b->sims[i]->ps, b->sims[i]->F, b->tun.tail_cells, &cg[i]);
+    limit = std::min(limit, b->sims[i]->cluster_limit);
   }
-  return exec_setup(b->ex, sd.data(), cg.data(), n, b->sims[0]->precision != 0, b->tun);
+  return exec_setup(b->ex, sd.data(), cg.data(), n, b->sims[0]->precision != 0, b->tun, limit);
 }
 
 // Device state of the simulations being tuned, copied aside so that every trial
@@ -848,7 +852,7 @@ int mdbs_create(const mdbs_grid* grid, const double* porosity, const double* per
     StepDom sd = step_view(s);
     CgDom cg;
     pressure_view(s->ps, s->F, s->tun.tail_cells, &cg);
-    e = exec_setup(s->ex, &sd, &cg, 1, s->precision != 0, s->tun);
+    e = exec_setup(s->ex, &sd, &cg, 1, s->precision != 0, s->tun, s->cluster_limit);
   }
   if (e == cudaSuccess) {
     Activate act(s);
@@ -1050,6 +1054,16 @@ int mdbs_set_tuning(mdbs_sim* s, const mdbs_tuning* t) {
     return cuda_fail(s, e, "set_tuning");
   }
   return MDBS_OK;
+}
+
+int mdbs_debug_cluster_limit(mdbs_sim* s, int32_t max_ctas) {
+  if (!s) return MDBS_ERR_ARG;
+  if (max_ctas < 0) return fail(s, MDBS_ERR_ARG, "max_ctas must be >= 0");
+  if (s->in_batch) return fail(s, MDBS_ERR_ARG, "the simulation belongs to a batch");
+  CK(cudaStreamSynchronize(s->stream));
+  s->cluster_limit = max_ctas;
+  const cudaError_t e = sim_exec_setup(s);
+  return e == cudaSuccess ? MDBS_OK : cuda_fail(s, e, "cluster_limit");
 }
 
 int mdbs_get_tuning(const mdbs_sim* s, mdbs_tuning* out) {

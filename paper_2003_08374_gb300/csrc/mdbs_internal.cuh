@@ -162,7 +162,7 @@ struct CgDom {
   Level<float> lf[kMaxLevels];   // FP32 hierarchy (mixed precision)
   int nlev;
   int first;  // first level handled by the tail kernel
-  int small;  // the whole CG solve runs in one cluster
+  int small;  // the whole CG solve may run in one cluster
   double *r, *z, *dv, *q;
   double* partials;  // 2 channels of pcap values
   long long pcap;
@@ -447,10 +447,14 @@ cudaError_t bounded_wait_selftest(int* status, double* waited_s);
 // sweep_kz: planes per fused-sweep chunk (0: half sweeps); tail_ctas: CTAs per domain
 // in the tail kernel (1, 2, 4, 8: one cluster)
 // coarse_coop: run the levels between the finest and the tail in one cooperative launch
+// cluster_limit: clusters of more CTAs than this count as ones the device cannot run
 cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexible, int smooth_rows, int snake,
-                        int sweep_kz, int tail_ctas, int coarse_coop, int vec_sweeps, BatchPlan* out);
-// launch shape of the cluster kernels (pressure.cu); n_small / n_big are set
-cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas, int sms, BatchPlan* B);
+                        int sweep_kz, int tail_ctas, int coarse_coop, int vec_sweeps, int cluster_limit,
+                        BatchPlan* out);
+constexpr int kClusterLimit = 16;  // the largest cluster there is: no limit
+// which domains the cluster kernels take (small[d]) and with what launch shape (pressure.cu)
+cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas, int sms, int cluster_limit,
+                          char* small, BatchPlan* B);
 // CTAs of the cooperative coarse-level kernel that are resident at once on this device
 cudaError_t coop_grid_size(int flexible, long long tail_words, int* grid);
 void plan_destroy(BatchPlan* B);

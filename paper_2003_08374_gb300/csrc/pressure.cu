@@ -2057,6 +2057,38 @@ cudaError_t bounded_wait_selftest(int* status, double* waited_s) {
   return e;
 }
 
+// the cluster kernel of a precision: rows cells a thread of the CG kernel, or (0) the tail
+static const void* cl_kernel(int flexible, int rows) {
+  if (rows == 0) return flexible ? (const void*)k_tail_cluster<float> : (const void*)k_tail_cluster<double>;
+  if (rows == 1) return flexible ? (const void*)k_cg_cluster<float, 1> : (const void*)k_cg_cluster<double, 1>;
+  if (rows == 2) return flexible ? (const void*)k_cg_cluster<float, 2> : (const void*)k_cg_cluster<double, 2>;
+  return flexible ? (const void*)k_cg_cluster<float, 4> : (const void*)k_cg_cluster<double, 4>;
+}
+
+// Clusters of ctas CTAs of that kernel that the device holds at once; 0: it cannot run one
+// (a cluster needs its SMs in one GPC: of 16 CTAs that fill an SM each a GB300 holds 7, and
+// a part with fewer SMs a GPC, or a partition of one, may hold none).
+static int cl_resident(int flexible, int rows, int ctas, size_t smem) {
+  if (smem > kClSmemMax) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, cl_kernel(flexible, rows), &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
 cudaError_t sweep_kernel_setup() {
   cudaError_t e =
       cudaFuncSetAttribute(k_smooth_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem_bytes());
@@ -2068,14 +2100,15 @@ cudaError_t sweep_kernel_setup() {
     e = cudaFuncSetAttribute(k_coarse_coop<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_coarse_coop<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMax);
-  const void* cl[] = {(const void*)k_tail_cluster<double>, (const void*)k_tail_cluster<float>,
-                      (const void*)k_cg_cluster<double, 1>, (const void*)k_cg_cluster<double, 2>,
-                      (const void*)k_cg_cluster<double, 4>, (const void*)k_cg_cluster<float, 1>,
-                      (const void*)k_cg_cluster<float, 2>, (const void*)k_cg_cluster<float, 4>};
-  for (const void* k : cl) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  }
+  // A device that refuses one of these runs no cluster of that kernel (cl_resident then
+  // finds none) and takes the launches instead.
+  for (int flexible = 0; flexible < 2 && e == cudaSuccess; flexible++)
+    for (int rows = 0; rows <= kClRowsMax; rows = rows ? 2 * rows : 1) {
+      const void* k = cl_kernel(flexible, rows);
+      cudaError_t c = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax);
+      if (c == cudaSuccess) c = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (c != cudaSuccess) cudaGetLastError();
+    }
   return e;
 }
 
@@ -2089,8 +2122,10 @@ static size_t tail_smem_bytes(const BatchPlan& B, size_t word, int ctas) {
 // Which domains the cluster kernels take and with what launch shape.  Small domains (every
 // level in the tail, at most kClCells cells) run their whole CG solve in a cluster; the
 // others' tails run in one when every tail starts at a level of at most kClCells cells.
-// More CTAs share a level's FP64 work; with many domains the GPU is full without.
-cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas, int sms, BatchPlan* B) {
+// More CTAs share a level's FP64 work; with many domains the GPU is full without.  Clusters
+// that the device cannot run give way to smaller ones, and these to the launches.
+cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas, int sms, int cluster_limit,
+                          char* small, BatchPlan* B) {
   auto ctas_for = [](long long cells, int per) {
     int c = 1;
     while ((long long)c * per < cells) c *= 2;
@@ -2101,41 +2136,63 @@ cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas
     return flexible ? cl_bytes<float>(cg[d].lf, first, cg[d].nlev, ctas, rows, 0)
                     : cl_bytes<double>(cg[d].ld, first, cg[d].nlev, ctas, rows, 0);
   };
-  bool tails = B->n_big > 0;
-  long long most_small = 1, most = 1;
+  auto runs = [&](int rows, int ctas, size_t smem) {
+    return ctas <= cluster_limit && cl_resident(flexible, rows, ctas, smem) > 0;
+  };
+  int n_small = 0;
+  long long most_small = 1;
   for (int d = 0; d < ndom; d++) {
-    if (cg[d].small) {
-      if (cg[d].ld[0].cells > most_small) most_small = cg[d].ld[0].cells;
-    } else {
-      const long long n = cg[d].ld[cg[d].first].cells;
-      if (cg[d].first == 0 || n > kClCells) tails = false;
-      if (n > most) most = n;
-    }
+    small[d] = cg[d].small;
+    if (!small[d]) continue;
+    n_small++;
+    if (cg[d].ld[0].cells > most_small) most_small = cg[d].ld[0].cells;
   }
-  // one reduction row a CTA while every CTA then has an SM of its own, else more
   auto small_for = [&](int rows) {
     if (most_small <= kClRow * rows) return 1;
     return (int)((most_small + kClSum - 1) / kClSum) * (kRepBig / rows);
   };
-  B->small_rows = 1;
-  while (B->small_rows < kClRowsMax && B->n_small * small_for(B->small_rows) > sms) B->small_rows *= 2;
-  for (;; B->small_rows /= 2) {
-    B->small_ctas = small_for(B->small_rows);
+  auto small_fits = [&](int rows) {
+    B->small_rows = rows;
+    B->small_ctas = small_for(rows);
     B->small_smem = 0;
     for (int d = 0; d < ndom; d++)
-      if (cg[d].small) B->small_smem = std::max(B->small_smem, bytes(d, 0, B->small_ctas, B->small_rows));
-    if (B->small_smem <= kClSmemMax || B->small_rows == 1) break;
+      if (small[d]) B->small_smem = std::max(B->small_smem, bytes(d, 0, B->small_ctas, rows));
+    return runs(rows, B->small_ctas, B->small_smem);
+  };
+  if (n_small > 0) {
+    // one reduction row a CTA while every CTA then has an SM of its own, else more
+    int rows = 1;
+    while (rows < kClRowsMax && n_small * small_for(rows) > sms) rows *= 2;
+    bool ok = false;
+    for (int r = rows; !ok && r <= kClRowsMax; r *= 2) ok = small_fits(r);  // the same cells in fewer CTAs
+    for (int r = rows / 2; !ok && r >= 1; r /= 2) ok = small_fits(r);       // less shared memory a CTA
+    if (!ok)
+      for (int d = 0; d < ndom; d++) small[d] = 0;
+  }
+  int n_big = 0;
+  long long most = 1;
+  bool tails = true;
+  for (int d = 0; d < ndom; d++) {
+    if (small[d]) continue;
+    const long long n = cg[d].ld[cg[d].first].cells;
+    if (cg[d].first == 0 || n > kClCells) tails = false;
+    if (n > most) most = n;
+    n_big++;
   }
   int ctas = 0;
-  if (tails) {
+  if (tails && n_big > 0) {
     ctas = tail_ctas > 1 ? tail_ctas : ctas_for(most, kClRow);
-    while (tail_ctas == 1 && ctas > 4 && ctas * B->n_big > sms) ctas /= 2;
+    while (tail_ctas == 1 && ctas > 4 && ctas * n_big > sms) ctas /= 2;
+    while (ctas > 0) {
+      B->cl_tail_smem = 0;
+      for (int d = 0; d < ndom; d++)
+        if (!small[d]) B->cl_tail_smem = std::max(B->cl_tail_smem, bytes(d, cg[d].first, ctas, 0));
+      if (runs(0, ctas, B->cl_tail_smem)) break;
+      ctas = tail_ctas == 1 && ctas > 4 && B->cl_tail_smem <= kClSmemMax ? ctas / 2 : 0;
+    }
   }
-  for (int d = 0; d < ndom; d++)
-    if (ctas && !cg[d].small) B->cl_tail_smem = std::max(B->cl_tail_smem, bytes(d, cg[d].first, ctas, 0));
-  if (B->cl_tail_smem > kClSmemMax) ctas = 0;
   B->cl_tail_ctas = ctas;
-  return B->small_smem <= kClSmemMax ? cudaSuccess : cudaErrorInvalidConfiguration;
+  return cudaSuccess;
 }
 
 cudaError_t coop_grid_size(int flexible, long long tail_words, int* grid) {

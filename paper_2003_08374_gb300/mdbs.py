@@ -116,6 +116,7 @@ def lib():
         L.mdbs_debug_array.argtypes = [C.c_void_p, C.c_char_p, _D, C.c_int64]
         L.mdbs_debug_array.restype = C.c_int64
         L.mdbs_check_bounded_wait.argtypes = [_D]
+        L.mdbs_debug_cluster_limit.argtypes = [C.c_void_p, C.c_int32]
         for nm in ("mdbs_set_tuning", "mdbs_get_tuning", "mdbs_batch_set_tuning", "mdbs_batch_get_tuning"):
             getattr(L, nm).argtypes = [C.c_void_p, C.POINTER(Tuning)]
         for nm in ("mdbs_autotune", "mdbs_batch_autotune"):
@@ -251,6 +252,10 @@ class Simulation:
         out = np.zeros(n)
         lib().mdbs_debug_array(self.h, name.encode(), _ptr(out), n)
         return out
+
+    def cluster_limit(self, max_ctas):
+        """Test aid: plan as on a device without clusters of more than max_ctas CTAs."""
+        self._check(lib().mdbs_debug_cluster_limit(self.h, int(max_ctas)))
 
     def set_stream(self, stream_handle: int):
         self._check(lib().mdbs_set_stream(self.h, C.c_void_p(stream_handle)))
