@@ -49,8 +49,9 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
     cudaError_t e = plan_clusters(cg, ndom, flexible, tail_ctas, sms, cluster_limit, small.data(), &B);
     if (e != cudaSuccess) return e;
   }
-  for (int d = 0; d < ndom; d++)
-    if (small[d]) idx[B.n_small++] = d;
+  for (int k = 0; k < B.n_shapes; k++)
+    for (int d = 0; d < ndom; d++)
+      if (small[d] == k + 1) idx[B.n_small++] = d;
   for (int d = 0; d < ndom; d++)
     if (!small[d]) idx[B.n_small + B.n_big++] = d;
   auto fill = [&](int space, auto count) -> int {

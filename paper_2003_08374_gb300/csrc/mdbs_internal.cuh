@@ -326,6 +326,13 @@ long long launch_count();  // kernels launched so far by the active simulation
   MDBS_LAUNCH_SMEM(ID, GRID, BLOCK, 0, STREAM, KERNEL, __VA_ARGS__)
 
 // ---------------------------------------------------------------- host-side batch plan
+// one launch of the CG cluster kernel: n domains, of lo < cells <= hi
+struct ClShape {
+  int n, rows, ctas;  // reduction rows per CTA, CTAs per cluster
+  long long lo, hi;
+  size_t smem;        // dynamic shared memory per CTA
+};
+
 // Block tables of one batch for every iteration space, uploaded once per
 // batch composition.
 struct BatchPlan {
@@ -336,8 +343,8 @@ struct BatchPlan {
   Work cgcells;               // CG vectors: kRepBig rows per item, domains solved by clusters left out
   int n_small, n_big;         // domains whose CG solve runs in a cluster, and the others
   const int *small_idx, *big_idx;  // device: their indexes
-  int small_rows, small_ctas; // reduction rows per CTA and CTAs per cluster of the CG kernel,
-  size_t small_smem;          // its dynamic shared memory
+  ClShape small[3];           // launches of the CG cluster kernel, largest domains first,
+  int n_shapes;               // over consecutive parts of small_idx
   int cl_tail_ctas;           // > 0: the tails run in clusters of this many CTAs
   size_t cl_tail_smem;
   Work lcells[kMaxLevels];    // level-l cells of domains that have level l, of more than kBuildCells cells
@@ -452,7 +459,8 @@ cudaError_t plan_create(const StepDom* sd, const CgDom* cg, int ndom, int flexib
                         int sweep_kz, int tail_ctas, int coarse_coop, int vec_sweeps, int cluster_limit,
                         BatchPlan* out);
 constexpr int kClusterLimit = 16;  // the largest cluster there is: no limit
-// which domains the cluster kernels take (small[d]) and with what launch shape (pressure.cu)
+// which domains the cluster kernels take (small[d]: 1 + the index of its launch in B->small;
+// 0: the launches) and with what launch shapes (pressure.cu)
 cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas, int sms, int cluster_limit,
                           char* small, BatchPlan* B);
 // CTAs of the cooperative coarse-level kernel that are resident at once on this device

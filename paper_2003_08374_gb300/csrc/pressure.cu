@@ -2136,38 +2136,92 @@ cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas
     return flexible ? cl_bytes<float>(cg[d].lf, first, cg[d].nlev, ctas, rows, 0)
                     : cl_bytes<double>(cg[d].ld, first, cg[d].nlev, ctas, rows, 0);
   };
-  auto runs = [&](int rows, int ctas, size_t smem) {
-    return ctas <= cluster_limit && cl_resident(flexible, rows, ctas, smem) > 0;
+  auto resident = [&](int rows, int ctas, size_t smem) {
+    return ctas <= cluster_limit ? cl_resident(flexible, rows, ctas, smem) : 0;
   };
-  int n_small = 0;
-  long long most_small = 1;
-  for (int d = 0; d < ndom; d++) {
-    small[d] = cg[d].small;
-    if (!small[d]) continue;
-    n_small++;
-    if (cg[d].ld[0].cells > most_small) most_small = cg[d].ld[0].cells;
-  }
-  auto small_for = [&](int rows) {
-    if (most_small <= kClRow * rows) return 1;
-    return (int)((most_small + kClSum - 1) / kClSum) * (kRepBig / rows);
-  };
-  auto small_fits = [&](int rows) {
-    B->small_rows = rows;
-    B->small_ctas = small_for(rows);
-    B->small_smem = 0;
+  // the launch of the small domains of lo < cells <= hi; *waves: how many times the clusters
+  // that the device holds at once it takes, *deep: most levels of these domains
+  auto shape_for = [&](long long lo, long long hi, int* waves, int* deep) {
+    ClShape S{};
+    S.lo = lo;
+    S.hi = hi;
+    long long most = 1;
+    *waves = *deep = 0;
+    auto in = [&](int d) { return cg[d].small && cg[d].ld[0].cells > lo && cg[d].ld[0].cells <= hi; };
     for (int d = 0; d < ndom; d++)
-      if (small[d]) B->small_smem = std::max(B->small_smem, bytes(d, 0, B->small_ctas, rows));
-    return runs(rows, B->small_ctas, B->small_smem);
-  };
-  if (n_small > 0) {
+      if (in(d)) {
+        S.n++;
+        most = std::max(most, (long long)cg[d].ld[0].cells);
+        *deep = std::max(*deep, cg[d].nlev);
+      }
+    if (S.n == 0) return S;
+    auto small_for = [&](int rows) {
+      if (most <= kClRow * rows) return 1;
+      return (int)((most + kClSum - 1) / kClSum) * (kRepBig / rows);
+    };
+    auto fits = [&](int rows) {
+      S.rows = rows;
+      S.ctas = small_for(rows);
+      S.smem = 0;
+      for (int d = 0; d < ndom; d++)
+        if (in(d)) S.smem = std::max(S.smem, bytes(d, 0, S.ctas, rows));
+      const int r = resident(rows, S.ctas, S.smem);
+      if (r > 0) *waves = (S.n + r - 1) / r;
+      return r > 0;
+    };
     // one reduction row a CTA while every CTA then has an SM of its own, else more
     int rows = 1;
-    while (rows < kClRowsMax && n_small * small_for(rows) > sms) rows *= 2;
+    while (rows < kClRowsMax && S.n * small_for(rows) > sms) rows *= 2;
     bool ok = false;
-    for (int r = rows; !ok && r <= kClRowsMax; r *= 2) ok = small_fits(r);  // the same cells in fewer CTAs
-    for (int r = rows / 2; !ok && r >= 1; r /= 2) ok = small_fits(r);       // less shared memory a CTA
-    if (!ok)
-      for (int d = 0; d < ndom; d++) small[d] = 0;
+    for (int r = rows; !ok && r <= kClRowsMax; r *= 2) ok = fits(r);  // the same cells in fewer CTAs
+    for (int r = rows / 2; !ok && r >= 1; r /= 2) ok = fits(r);       // less shared memory a CTA
+    if (!ok) S.n = 0;
+    return S;
+  };
+  // Where the cluster solve is the better one.  With one or two CTAs a domain it was at any
+  // count (a step of 512 x 2000 cells of a column 12.0 ms as launches, 10.1 in clusters; 512 x
+  // 12^3 5.4 / 5.4; 2048 x 256 16.4 / 9.5).  With more, a domain's share of the SMs' time is up
+  // against launches that fill the GPU: FP64, four CTAs, better up to three waves (100 x 64^2
+  // 2.64 / 2.36; 152: 3.31 / 3.70), eight, the least for grids of many levels, up to four (38 x
+  // 4096 5.39 / 3.51, 70: 5.80 / 5.93, 152: 7.02 / 11.5); FP32, whose launches are bound by
+  // latency for longer, up to four (130 x 64^2 2.78 / 2.60, 152: 3.00 / 3.12).  In FP32, eight or
+  // more such domains of few levels beside larger ones, whose launches run anyway, are cheaper
+  // there (8 x 16^3 + 8 x 24^3 1.91 / 2.08 ms; FP64 even).
+  bool others = false;
+  for (int d = 0; d < ndom; d++) others |= !cg[d].small;
+  auto better = [&](const ClShape& S, int waves, int deep) {
+    if (S.ctas <= 2) return true;
+    if (flexible && others && deep <= 8 && S.n >= 8) return false;
+    return waves <= (flexible || S.ctas > 4 ? 4 : 3);
+  };
+  // All small domains in one launch, shaped by the largest; or one launch for those of each
+  // size that takes the same CTAs, one after the other, where these are fewer waves in all
+  // (1 x 64^2 + 500 x 100 cells: 14 waves 5.5 ms, 1 + 4 waves 2.7).
+  const long long size[4] = {kClCells, kClSum, kClRow * kClRowsMax, 0};
+  int waves = 0, deep = 0, parts = 0, part_waves = 0;
+  ClShape part[3];
+  bool part_ok[3];
+  const ClShape one = shape_for(0, kClCells, &waves, &deep);
+  for (int k = 0; k < 3; k++) {
+    int pw = 0, pd = 0;
+    const ClShape S = shape_for(size[k + 1], size[k], &pw, &pd);
+    if (S.n == 0) continue;
+    part[parts] = S;
+    part_ok[parts++] = better(S, pw, pd);
+    part_waves += pw;
+  }
+  B->n_shapes = 0;
+  if (one.n > 0 && (parts <= 1 || waves <= part_waves) && better(one, waves, deep)) {
+    B->small[B->n_shapes++] = one;
+  } else {
+    for (int k = 0; k < parts; k++)
+      if (part_ok[k]) B->small[B->n_shapes++] = part[k];
+  }
+  for (int d = 0; d < ndom; d++) {
+    small[d] = 0;
+    for (int k = 0; k < B->n_shapes; k++)
+      if (cg[d].small && cg[d].ld[0].cells > B->small[k].lo && cg[d].ld[0].cells <= B->small[k].hi)
+        small[d] = (char)(k + 1);
   }
   int n_big = 0;
   long long most = 1;
@@ -2187,7 +2241,7 @@ cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas
       B->cl_tail_smem = 0;
       for (int d = 0; d < ndom; d++)
         if (!small[d]) B->cl_tail_smem = std::max(B->cl_tail_smem, bytes(d, cg[d].first, ctas, 0));
-      if (runs(0, ctas, B->cl_tail_smem)) break;
+      if (resident(0, ctas, B->cl_tail_smem) > 0) break;
       ctas = tail_ctas == 1 && ctas > 4 && B->cl_tail_smem <= kClSmemMax ? ctas / 2 : 0;
     }
   }
@@ -2696,21 +2750,22 @@ cudaError_t pressure_solve(const BatchPlan& B, double tol, int max_it, int nu1, 
                            bool capture, cudaStream_t s, cudaStream_t body_stream, double* host_flag,
                            long long* body_launches) {
   const int flexible = B.flexible;  // the hierarchy comes from launch_pressure_matrix
-  if (B.n_small > 0) {
+  for (int k = 0, at = 0; k < B.n_shapes; k++) {
+    const ClShape& S = B.small[k];
     prof_begin(K_CG_CLUSTER, s);
     auto launch = [&](auto kernel) {
-      return launch_cluster(kernel, B.n_small, B.small_ctas, B.small_smem, s, B.sd, B.cg, B.small_idx, B.small_ctas, nu1,
-                            nu2, cs, tol, max_it, corr > 0 ? 1 : 0);
+      return launch_cluster(kernel, S.n, S.ctas, S.smem, s, B.sd, B.cg, B.small_idx + at, S.ctas, nu1, nu2, cs, tol,
+                            max_it, corr > 0 ? 1 : 0);
     };
-    const int rows = B.small_rows;
-    const cudaError_t le = flexible ? (rows == 1   ? launch(k_cg_cluster<float, 1>)
-                                       : rows == 2 ? launch(k_cg_cluster<float, 2>)
-                                                   : launch(k_cg_cluster<float, 4>))
-                                    : (rows == 1   ? launch(k_cg_cluster<double, 1>)
-                                       : rows == 2 ? launch(k_cg_cluster<double, 2>)
-                                                   : launch(k_cg_cluster<double, 4>));
+    const cudaError_t le = flexible ? (S.rows == 1   ? launch(k_cg_cluster<float, 1>)
+                                       : S.rows == 2 ? launch(k_cg_cluster<float, 2>)
+                                                     : launch(k_cg_cluster<float, 4>))
+                                    : (S.rows == 1   ? launch(k_cg_cluster<double, 1>)
+                                       : S.rows == 2 ? launch(k_cg_cluster<double, 2>)
+                                                     : launch(k_cg_cluster<double, 4>));
     if (le != cudaSuccess) set_launch_error(le);
     prof_end(K_CG_CLUSTER, s);
+    at += S.n;
   }
   if (B.n_big == 0) {
     if (body_launches) *body_launches = 0;
