@@ -2235,14 +2235,27 @@ cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas
   }
   int ctas = 0;
   if (tails && n_big > 0) {
-    ctas = tail_ctas > 1 ? tail_ctas : ctas_for(most, kClRow);
-    while (tail_ctas == 1 && ctas > 4 && ctas * n_big > sms) ctas /= 2;
-    while (ctas > 0) {
+    // clusters of c CTAs that the device holds at once
+    auto tail_resident = [&](int c) {
       B->cl_tail_smem = 0;
       for (int d = 0; d < ndom; d++)
-        if (!small[d]) B->cl_tail_smem = std::max(B->cl_tail_smem, bytes(d, cg[d].first, ctas, 0));
-      if (resident(0, ctas, B->cl_tail_smem) > 0) break;
-      ctas = tail_ctas == 1 && ctas > 4 && B->cl_tail_smem <= kClSmemMax ? ctas / 2 : 0;
+        if (!small[d]) B->cl_tail_smem = std::max(B->cl_tail_smem, bytes(d, cg[d].first, c, 0));
+      return resident(0, c, B->cl_tail_smem);
+    };
+    // As many CTAs as there are rows of kClRow cells, or a half or a quarter of them, while all
+    // the clusters run at once on at most one and a half CTAs an SM; a second round of clusters
+    // or CTAs of many cells each cost more than the one CTA a domain of k_tail_vcycle (a step of
+    // 38 x 32^3 cells FP64 5.89 ms in clusters, 5.55 there; 128 x 100^2 8.6 / 6.6; FP32 76 x 5000
+    // 8.8 / 6.1; 8 x 5000 with 16 CTAs 4.96, 8 CTAs 4.13; 34 x 100^2 with 8 CTAs 3.51, 4 CTAs
+    // 3.02).  In FP64, whose arithmetic that one CTA runs on a single SM's pipe, eight CTAs a
+    // domain stay ahead up to the SMs' number (17 x 100^2 2.45 / 2.68).
+    if (tail_ctas > 1) {
+      if (tail_resident(tail_ctas) > 0) ctas = tail_ctas;
+    } else {
+      const int natural = ctas_for(most, kClRow), least = std::min(natural, 4);
+      for (int c = natural; !ctas && c >= least; c /= 2)
+        if ((c == least || 2 * c * n_big <= 3 * sms) && tail_resident(c) >= n_big) ctas = c;
+      if (!ctas && !flexible && natural >= 8 && 8 * n_big <= sms && tail_resident(8) > 0) ctas = 8;
     }
   }
   B->cl_tail_ctas = ctas;

@@ -21,6 +21,10 @@ BATCHES = {
     "many": [(16, 16, 16)] * 120,
     # many levels: the launches for these, clusters for the short ones
     "deep": [(2, 2048, 1)] * 40 + [(50, 1, 1)] * 7,
+    # tails of larger domains: clusters of four CTAs, of fewer than their rows, and too many
+    "tails_at_once": [(20, 17, 13)] * 30,
+    "tails_halved": [(33, 31, 17)] * 20,
+    "tails_many": [(20, 17, 13), (70, 70, 1)] * 40,
     # small domains that join the launches of a larger one (FP32)
     "beside": [(16, 16, 16)] * 9 + [(20, 20, 13)] + [(300, 1, 1)] * 3,
 }
