@@ -139,6 +139,7 @@ struct mdbs_sim {
   long long pcap;
   double* scal;       // device step scalars (kSlot* in mdbs_internal.cuh)
   double* host_scal;  // pinned copy of scal
+  cudaEvent_t ev_order = nullptr;  // mdbs_set_fields: the work queued ahead of it
   mdbs_stats st;
   double alpha_lo_seen = 0.0, alpha_hi_seen = 1.0;  // extremes of alpha this simulation's steps produced
   bool fields_set;
@@ -835,12 +836,14 @@ int mdbs_create(const mdbs_grid* grid, const double* porosity, const double* per
   cudaMemset(s->arena, 0, s->arena_bytes);
   carve(s, L, (char*)s->arena);
   e = cudaMallocHost(&s->host_scal, kNumSlots * sizeof(double));
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_order, cudaEventDisableTiming);
   if (e == cudaSuccess) s->ps = pressure_create(P, s->precision, &e);
   if (e != cudaSuccess) {
     int code = e == cudaErrorMemoryAllocation ? MDBS_ERR_OOM : MDBS_ERR_CUDA;
     fail(nullptr, code, std::string("pressure solver: ") + cudaGetErrorString(e));
     cudaGetLastError();
     if (s->host_scal) cudaFreeHost(s->host_scal);
+    if (s->ev_order) cudaEventDestroy(s->ev_order);
     dev_block_free(&s->arena_mem);
     delete s;
     return code;
@@ -892,22 +895,25 @@ int mdbs_set_fields(mdbs_sim* s, const double* alpha, const double* ux, const do
   // alpha goes to the low-order saturation scratch (which the next step overwrites), and only
   // an accepted field is copied into place, so a rejected call leaves the state unchanged.
   // The check runs on the device, in the order of the stream, where a kernel flags any value
-  // out of range, except for small fields in pageable memory: up to kHostCheck cells that
-  // array is read here, without the kernel, the flag's way back and a wait.  The copy below
-  // reads pageable memory when it is called; memory the runtime knows (pinned, managed) may
-  // be filled by work queued ahead of the copy, so its values are not yet there to be read.
-  // (The whole call, device -> host check: 2000 cells 88 -> 66 us, 8192 126 -> 98, 16384
-  // 121 -> 116, where the reading costs what the wait does.)
+  // out of range, except for small fields in host memory: up to kHostCheck cells the array is
+  // read here, without the kernel and the flag's way back.  The copy below reads pageable
+  // memory when it is called; a pinned array may be filled by work queued ahead of the copy, so
+  // it is read once an event recorded there has passed.  (The whole call, device -> host
+  // check, 2000 / 8192 / 16384 cells: pinned 81 -> 74, 87 -> 80, 90 -> 88 us; pageable 89 -> 67,
+  // 126 -> 96, 123 -> 113.)
   constexpr long long kHostCheck = 16384;
   const double lo = std::min(-1e-9, s->alpha_lo_seen), hi = std::max(1.0 + 1e-9, s->alpha_hi_seen);
   double* stage = s->F.aL;
-  CK(cudaMemcpyAsync(stage, alpha, s->P.cells * 8, cudaMemcpyHostToDevice, s->stream));
-  bool bad = false, host = false;
+  bool bad = false, host = false, pinned = false;
   if (s->P.cells <= kHostCheck) {
     cudaPointerAttributes at;
     CK(cudaPointerGetAttributes(&at, alpha));
-    host = at.type == cudaMemoryTypeUnregistered;
+    pinned = at.type == cudaMemoryTypeHost;
+    host = pinned || at.type == cudaMemoryTypeUnregistered;
+    if (pinned) CK(cudaEventRecord(s->ev_order, s->stream));
   }
+  CK(cudaMemcpyAsync(stage, alpha, s->P.cells * 8, cudaMemcpyHostToDevice, s->stream));
+  if (pinned) CK(cudaEventSynchronize(s->ev_order));
   if (host) {
     for (long long c = 0; c < s->P.cells; c++) bad |= !(alpha[c] >= lo && alpha[c] <= hi);
     if (bad) CK(cudaStreamSynchronize(s->stream));  // the copy has left the caller's array
@@ -984,6 +990,7 @@ void mdbs_destroy(mdbs_sim* s) {
   cudaDeviceSynchronize();
   exec_destroy(s->ex);
   pressure_destroy(s->ps);
+  if (s->ev_order) cudaEventDestroy(s->ev_order);
   if (s->host_scal) cudaFreeHost(s->host_scal);
   dev_block_free(&s->arena_mem);
   delete s;
