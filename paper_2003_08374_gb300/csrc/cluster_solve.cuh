@@ -137,23 +137,25 @@ __host__ __device__ inline int cl_children(const int cz[3], int mask) {
   return mask && n > 1 ? n / 2 : n;
 }
 
-// shared memory by 32-bit address: this CTA's (sh_) or any CTA's of the cluster (cl_)
+// Shared memory by 32-bit address: this CTA's (sh_) or any CTA's of the cluster (cl_).  The
+// loads clobber memory as the stores do: some of it (the level table, the exchanged sums) is
+// also read or written by C++ statements, which the compiler may then not move past them.
 __device__ __forceinline__ unsigned sh_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned cl_map(unsigned addr, unsigned rank) {
   unsigned r;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void sh_ld(unsigned a, double& v) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a)); }
-__device__ __forceinline__ void sh_ld(unsigned a, float& v) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a)); }
+__device__ __forceinline__ void sh_ld(unsigned a, double& v) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory"); }
+__device__ __forceinline__ void sh_ld(unsigned a, float& v) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory"); }
 __device__ __forceinline__ unsigned sh_ldw(unsigned a) {
   unsigned v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
   return v;
 }
 __device__ __forceinline__ unsigned sh_ld16(unsigned a) {
   unsigned short v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
   return v;
 }
 __device__ __forceinline__ void sh_st(unsigned a, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
@@ -170,14 +172,14 @@ __device__ __forceinline__ void sh_st_if(unsigned a, float v, bool ok) {
   asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.shared.f32 [%0], %1;\n}\n" ::"r"(a), "f"(v), "r"((unsigned)ok) : "memory");
 }
 __device__ __forceinline__ void cl_ld(unsigned a, double& v) {
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
 }
 __device__ __forceinline__ void cl_ld(unsigned a, float& v) {
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
 }
 __device__ __forceinline__ unsigned cl_ld16(unsigned a) {
   unsigned short v;
-  asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(a));
+  asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
   return v;
 }
 __device__ __forceinline__ void cl_st(unsigned a, double v) {
@@ -197,11 +199,13 @@ __device__ __forceinline__ void cl_wait() {
 // phases of the cluster that is an arrival at the cluster barrier, which the next phase
 // (or whoever reads the result) waits for.
 //
-// Who runs a phase is a template parameter and each phase has one or two call sites, so
-// that everything is inlined.  (As functions of their own they were no faster, and with four
-// rows a CTA, where caller and callee together are short of registers, nvcc 13.0 built a
-// kernel whose results were wrong on one shape, 9 x 20 x 11.)  They take shared addresses
-// (lv: a ClLevel), so nothing lives in local memory.
+// Who runs a phase is a template parameter, and every phase is inlined.  As functions of
+// their own they were no faster, and gave wrong results, not the same ones each time, with
+// four rows a CTA in FP64 on 9 x 20 x 11 cells.  The cause of that is not known: reading the
+// phases' barriers for that shape showed none, and the loads above did not clobber memory
+// then.  The inlined form is compared bit for bit with the launches over shapes of every row
+// count.  The phases take shared addresses (lv: a ClLevel) and copy no table to local memory;
+// what the four-row FP64 kernel holds there is 136 bytes of spilled registers.
 enum { kByCluster = 0, kByBlock = 1, kByWarp = 2 };
 template <int KIND>
 __device__ __forceinline__ void cl_begin() {
