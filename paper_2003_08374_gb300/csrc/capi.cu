@@ -23,7 +23,7 @@ namespace mdbs {
 const char* const kKernelNames[K_COUNT] = {
     "alpha_flux", "alpha_lo", "alpha_limit", "alpha_update", "finalize", "properties", "normals",
     "curvature", "momentum_assemble", "jacobi", "hbya", "correct", "boundary", "field_stats", "cfl",
-    "static_geometry", "pressure_assemble", "diag", "convert", "coarsen", "smooth_fine", "smooth_coarse",
+    "static_geometry", "pressure_assemble", "coarsen", "smooth_fine", "smooth_coarse",
     "zero", "restrict_fine", "restrict_coarse", "prolong_fine", "prolong_coarse", "cg_resid0",
     "cg_spmv_dot", "cg_update_xr", "cg_dots", "cg_update_d", "tail_vcycle", "coarse_coop", "edge_viscosity", "cg_cluster"};
 

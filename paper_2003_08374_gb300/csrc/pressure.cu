@@ -122,7 +122,7 @@ __device__ __forceinline__ void with_coefs(const Level<R>& L, F&& f) {
 }
 
 // CG scalars on the device
-constexpr int kBB = 0, kRR = 1, kRZ = 2, kDQ = 3, kZQ = 4, kAlpha = 5, kCond = 6, kBeta = 7, kIt = 8;
+constexpr int kBB = 0, kRR = 1, kRZ = 2, kAlpha = 3, kCond = 4, kBeta = 5, kIt = 6;
 
 #define FOR_WORK(W)                                   \
   for (int b_ = blockIdx.x; b_ < (W).total; b_ += gridDim.x) { \
@@ -1866,7 +1866,6 @@ __global__ void k_update_d(const __grid_constant__ CgVec one, const CgVec* __res
 // The loop condition "not converged, below max_it, finite" goes to scal[kCond].
 __device__ __forceinline__ void cg_scalars(double* scal, int mode, int two, double a, double b, double tol, int max_it) {
   if (mode == 1) {
-    scal[kDQ] = a;
     scal[kAlpha] = scal[kRZ] / a;
   } else if (mode == 3) {
     const double old = scal[kRZ];
