@@ -239,11 +239,12 @@ void mdbs_batch_destroy(mdbs_batch* batch);
  *                 coarser ones, inside one kernel (fewer launches, less parallelism).
  *                 Where that starts at a level of at most 4096 cells in every domain,
  *                 the kernel is a thread-block cluster per domain that keeps the levels
- *                 in its shared memory; a domain that lies wholly in it, of at most
- *                 4096 cells, runs its whole CG solve there
+ *                 in its shared memory, while the device can run all of these at once;
+ *                 a domain that lies wholly in it, of at most 4096 cells, runs its whole
+ *                 CG solve there, while that is the faster way for the batch
  *   tail_ctas   : 1, 2, 4 or 8; CTAs per domain in that kernel (more than one: a
  *                 thread-block cluster synchronised by cluster barriers); 1 leaves the
- *                 size of the clusters above to the library
+ *                 size and use of the clusters above to the library
  *   snake       : 0 or 1; 1 alternates the traversal direction of consecutive
  *                 kernels over one level, so each starts on the cache lines the
  *                 previous one touched last

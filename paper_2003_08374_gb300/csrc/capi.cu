@@ -662,9 +662,8 @@ int autotune_impl(const std::vector<mdbs_sim*>& sims, Exec& ex, const mdbs_optio
   const int rows[] = {1, 2, 4, 8};
   const int coops[] = {0, 1};
   const int vecs[] = {0, 1};
-  // (tail_cells, tail_ctas): larger tails want more CTAs
-  // (1024: a 2-D grid's 32^2 level; the 64^2 fracture case measured 1.18 against 1.35 ms per
-  // step with its whole V-cycle in one CTA)
+  // (tail_cells, tail_ctas): larger tails want more CTAs (up to 4096 cells 1 leaves them to the
+  // plan; 1024: a 2-D grid's 32^2 level)
   const int tails[][2] = {{0, 1}, {512, 1}, {1024, 1}, {4096, 1}, {4096, 4}, {32768, 4}, {32768, 8}, {262144, 8}};
   for (int axis = 0; axis < 6 && e == cudaSuccess; axis++) {
     if (axis == 2 && best.sweep_kz > 0 && fp32_levels) continue;

@@ -832,9 +832,9 @@ __global__ void __launch_bounds__(kClThreads, 2)
   Cl<R> c{sh_addr(lv), blockIdx.x % ctas, 0u};
   unsigned end;
   const int first = G.first, nlev = G.nlev;
-  // Before the wait on the preceding kernel (a restriction or a half sweep): everything the
-  // setup reads was written by the operator's build, which had completed before that
-  // kernel passed its own wait.
+  // Before the wait on the preceding kernel (a restriction or a half sweep, which may not have
+  // waited itself): everything the setup reads was written by the operator's build, which had
+  // completed before any kernel of the loop started (MDBS_PDL_TRIGGER).
   cl_setup<R>(c, lv, gl, sh_addr(cl_sm), G, first, nlev, ctas, 0, nu1 > 0 ? 1 : 0, &end);
   MDBS_DEPENDENT_ENTRY();
   // every thread of the cluster has left the setup's remote reads of res behind
@@ -881,7 +881,8 @@ __global__ void __launch_bounds__(kClThreads, 1)
   // A step's first solve waits here: the operator's build may be among the kernels it follows
   // (the branch it runs on joins ahead of this kernel, and a captured join can be a
   // programmatic dependency like any other).  In the later ones, which follow the first, the
-  // setup overlaps the preceding kernel; all it reads is the operator.
+  // setup overlaps the preceding kernel (another size's solve among them); all it reads is the
+  // operator.
   if (!early) MDBS_PDL_WAIT();
   cl_setup<R>(c, lv, gl, sh_addr(cl_sm), G, 0, nlev, ctas, ROWS, nu1 > 0 ? 1 : 0, &end);
   const unsigned db = end;  // the vector A is applied to, exchanged through the cluster

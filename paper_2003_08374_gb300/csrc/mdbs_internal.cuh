@@ -284,22 +284,25 @@ long long launch_count();  // kernels launched so far by the active simulation
 
 //
 // Launches are programmatic dependent launches: a kernel may be scheduled while
-// its predecessor in the stream drains, and every kernel begins with
-// MDBS_DEPENDENT_ENTRY(), which waits until the predecessor grid has completed and
-// its memory is visible (griddepcontrol.wait) before touching any data, then lets
-// its own successor start launching (griddepcontrol.launch_dependents).  The
-// order of all memory effects is therefore the plain stream order; only the launch
-// latency between dependent kernels overlaps (also inside captured graphs).
+// its predecessor in the stream drains.  Every kernel waits until the predecessor
+// grid has completed and its memory is visible (griddepcontrol.wait) before it
+// touches anything that a kernel of the step rewrites, and lets its own successor
+// start launching (griddepcontrol.launch_dependents).  All but the kernels of the CG
+// loop do both first thing, with MDBS_DEPENDENT_ENTRY().  The order of all memory
+// effects is therefore the plain stream order; only the launch latency between
+// dependent kernels overlaps (also inside captured graphs).
 #define MDBS_DEPENDENT_ENTRY()                                    \
   do {                                                            \
     asm volatile("griddepcontrol.wait;\n" ::: "memory");          \
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); \
   } while (0)
 
-// The two halves apart, for the kernels of the CG loop: they let their successor launch at
-// once and read what no kernel of the loop writes (tables, coefficients, reciprocal
-// diagonals: written by the operator's build, which has completed before the loop's first
-// kernel starts) before they wait.  A kernel that has not waited may run beside any number
+// The two halves apart, for the kernels of the CG loop, which let their successor launch at
+// once.  k_sweep and k_resid_restrict of a single domain, k_tail_cluster, and k_cg_cluster in
+// a step's later solves read the operator (tables, coefficients, reciprocal diagonals,
+// coarsest inverse) before they wait: no kernel of the loop writes it, and its build has
+// completed before any kernel of the loop starts, because the kernels ahead of the loop wait
+// before they let a successor launch.  A kernel that has not waited may run beside any number
 // of its predecessors, so it must touch nothing else.
 #define MDBS_PDL_TRIGGER() asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory")
 #define MDBS_PDL_WAIT() asm volatile("griddepcontrol.wait;\n" ::: "memory")
