@@ -2139,19 +2139,18 @@ cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas
     return ctas <= cluster_limit ? cl_resident(flexible, rows, ctas, smem) : 0;
   };
   // the launch of the small domains of lo < cells <= hi; *waves: how many times the clusters
-  // that the device holds at once it takes, *deep: most levels of these domains
-  auto shape_for = [&](long long lo, long long hi, int* waves, int* deep) {
+  // that the device holds at once it takes
+  auto shape_for = [&](long long lo, long long hi, int* waves) {
     ClShape S{};
     S.lo = lo;
     S.hi = hi;
     long long most = 1;
-    *waves = *deep = 0;
+    *waves = 0;
     auto in = [&](int d) { return cg[d].small && cg[d].ld[0].cells > lo && cg[d].ld[0].cells <= hi; };
     for (int d = 0; d < ndom; d++)
       if (in(d)) {
         S.n++;
         most = std::max(most, (long long)cg[d].ld[0].cells);
-        *deep = std::max(*deep, cg[d].nlev);
       }
     if (S.n == 0) return S;
     auto small_for = [&](int rows) {
@@ -2184,33 +2183,45 @@ cudaError_t plan_clusters(const CgDom* cg, int ndom, int flexible, int tail_ctas
   // 2.64 / 2.36; 152: 3.31 / 3.70), eight, the least for grids of many levels, up to four (38 x
   // 4096 5.39 / 3.51, 70: 5.80 / 5.93, 152: 7.02 / 11.5); FP32, whose launches are bound by
   // latency for longer, up to four (130 x 64^2 2.78 / 2.60, 152: 3.00 / 3.12).  In FP32, eight or
-  // more such domains of few levels beside larger ones, whose launches run anyway, are cheaper
-  // there (8 x 16^3 + 8 x 24^3 1.91 / 2.08 ms; FP64 even).
-  bool others = false;
-  for (int d = 0; d < ndom; d++) others |= !cg[d].small;
-  auto better = [&](const ClShape& S, int waves, int deep) {
+  // more domains of more than kClSum cells and few levels are cheaper in the launches of larger
+  // ones, which run anyway (8 x 16^3 + 8 x 24^3 1.91 / 2.08 ms; FP64 even), unless smaller ones
+  // run in clusters anyway, too (9 x 16^3 + 20 x 300 + 24^3 2.01 / 1.86).
+  bool others = false, narrow = false;
+  int wide = 0, wide_deep = 0;  // small domains of more than kClSum cells, and their most levels
+  for (int d = 0; d < ndom; d++) {
+    if (!cg[d].small) {
+      others = true;
+    } else if (cg[d].ld[0].cells <= kClSum) {
+      narrow = true;
+    } else {
+      wide++;
+      wide_deep = std::max(wide_deep, cg[d].nlev);
+    }
+  }
+  const bool join = flexible && others && !narrow && wide >= 8 && wide_deep <= 8;
+  auto better = [&](const ClShape& S, int waves) {
     if (S.ctas <= 2) return true;
-    if (flexible && others && deep <= 8 && S.n >= 8) return false;
+    if (join) return false;
     return waves <= (flexible || S.ctas > 4 ? 4 : 3);
   };
   // All small domains in one launch, shaped by the largest; or one launch for those of each
   // size that takes the same CTAs, one after the other, where these are fewer waves in all
   // (1 x 64^2 + 500 x 100 cells: 14 waves 5.5 ms, 1 + 4 waves 2.7).
   const long long size[4] = {kClCells, kClSum, kClRow * kClRowsMax, 0};
-  int waves = 0, deep = 0, parts = 0, part_waves = 0;
+  int waves = 0, parts = 0, part_waves = 0;
   ClShape part[3];
   bool part_ok[3];
-  const ClShape one = shape_for(0, kClCells, &waves, &deep);
+  const ClShape one = shape_for(0, kClCells, &waves);
   for (int k = 0; k < 3; k++) {
-    int pw = 0, pd = 0;
-    const ClShape S = shape_for(size[k + 1], size[k], &pw, &pd);
+    int pw = 0;
+    const ClShape S = shape_for(size[k + 1], size[k], &pw);
     if (S.n == 0) continue;
     part[parts] = S;
-    part_ok[parts++] = better(S, pw, pd);
+    part_ok[parts++] = better(S, pw);
     part_waves += pw;
   }
   B->n_shapes = 0;
-  if (one.n > 0 && (parts <= 1 || waves <= part_waves) && better(one, waves, deep)) {
+  if (one.n > 0 && (parts <= 1 || waves <= part_waves) && better(one, waves)) {
     B->small[B->n_shapes++] = one;
   } else {
     for (int k = 0; k < parts; k++)

@@ -25,7 +25,8 @@ BATCHES = {
     "tails_at_once": [(20, 17, 13)] * 30,
     "tails_halved": [(33, 31, 17)] * 20,
     "tails_many": [(20, 17, 13), (70, 70, 1)] * 40,
-    # small domains that join the launches of a larger one (FP32)
+    # small domains that join the launches of a larger one (FP32), and that do not
+    "joined": [(16, 16, 16)] * 9 + [(20, 20, 13)],
     "beside": [(16, 16, 16)] * 9 + [(20, 20, 13)] + [(300, 1, 1)] * 3,
 }
 
